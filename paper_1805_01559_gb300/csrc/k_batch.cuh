@@ -171,6 +171,7 @@ __device__ __noinline__ bool bt_instance(const BInst& D, BRes* out, int* abort, 
         mbar_fence_init();
     }
     __shared__ int s_res;
+    if (warp == 0) tmem_alloc(&sh->tmem, tmem_cols<1, VPT>());
     __syncthreads();
     if (warp == BT_NCW) {
         if (lane == 0) stream_rows_producer(P.C, P.ld, r0, r1, S, ring, full, empty, &sh->s_stop, abort, spin);
@@ -187,6 +188,7 @@ __device__ __noinline__ bool bt_instance(const BInst& D, BRes* out, int* abort, 
         }
     }
     __syncthreads();  // the producer has drained its copies
+    if (warp == 0) tmem_free(sh->tmem, tmem_cols<1, VPT>());
     if (ld_volatile_i32(abort) != DEV_OK) return false;
     if (s_res == 0) {  // the instance failed (the same in every CTA of the group)
         if (rank == 0 && threadIdx.x == 0) {

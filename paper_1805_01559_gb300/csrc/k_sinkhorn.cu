@@ -36,100 +36,10 @@
 #include "ot_common.cuh"
 #include "sk_core.cuh"
 #include "sk_multi.cuh"
+#include "sk_kernels.cuh"
 #include "ot_internal.h"
 
 namespace ota {
-
-template <int TW, int VPT>
-__global__ void __launch_bounds__(Cons<TW>::NT, 1) sk_solve(SolveParams P, StreamCfg S) {
-    constexpr int NCW = Cons<TW>::NCW;
-    extern __shared__ __align__(128) unsigned char dyn[];
-    __shared__ SkShared sh;
-    uint64_t* full = reinterpret_cast<uint64_t*>(dyn);
-    uint64_t* empty = full + MAX_STAGES;
-    float* ring = reinterpret_cast<float*>(dyn + S.off_ring);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int64_t r0, r1;
-    cta_rows(P.I, S.rows_per_stage, P.V, blockIdx.x, gridDim.x, &r0, &r1);
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S.stages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], NCW);
-        }
-        sh.s_stop = 0;
-        sh.s_bad = 0;
-        mbar_fence_init();
-    }
-    __syncthreads();
-    if (warp == NCW) {
-        if (lane == 0)
-            stream_rows_producer(P.C, P.ld, r0, r1, S, ring, full, empty, &sh.s_stop, &P.st->status, P.spin);
-        return;
-    }
-    GroupCtx g{(int)gridDim.x, (int)blockIdx.x, &P.st->bar, 0u, &P.st->status, &P.st->status};
-    int par = 0;
-    sk_consumers<TW, VPT>(P, S, g, &sh, dyn, r0, r1, &par);
-}
-
-// Euclidean cost formed on the fly (Sec. IV cost choice (i)): no matrix is read, so there is
-// no producer warp (the block is the consumer warps alone, which leaves each thread more
-// registers); the RRH coordinates are staged once in the ring's space and every sweep forms
-// C_ij = ||x_i - x_j|| from them and the device's coordinates.
-template <int TW, int VPT>
-__global__ void __launch_bounds__(Cons<TW>::NCW * 32, 1) sk_solve_euclid(SolveParams P, StreamCfg S) {
-    constexpr int NCW = Cons<TW>::NCW;
-    extern __shared__ __align__(128) unsigned char dyn[];
-    __shared__ SkShared sh;
-    float* rx = reinterpret_cast<float*>(dyn + S.off_ring);
-    for (int j = threadIdx.x; j < P.Jp; j += blockDim.x) {
-        const float2 r = j < P.J ? P.rrh_xy[j] : make_float2(0.f, 0.f);
-        rx[j] = r.x;
-        rx[P.Jp + j] = r.y;
-    }
-    if (threadIdx.x == 0) {
-        sh.s_stop = 0;
-        sh.s_bad = 0;
-    }
-    __syncthreads();
-    int64_t r0, r1;
-    cta_rows(P.I, S.rows_per_stage, P.V, blockIdx.x, gridDim.x, &r0, &r1);
-    GroupCtx g{(int)gridDim.x, (int)blockIdx.x, &P.st->bar, 0u, &P.st->status, &P.st->status};
-    int par = 0;
-    sk_consumers<TW, VPT, true>(P, S, g, &sh, dyn, r0, r1, &par);
-}
-
-// Several solves sharing one cost matrix (sk_multi.cuh): the same launch structure.
-template <int TW, int VPT, int NS, bool RC>
-__global__ void __launch_bounds__(Cons<TW>::NT, 1) sk_solve_multi(MultiParams M, StreamCfg S) {
-    constexpr int NCW = Cons<TW>::NCW;
-    extern __shared__ __align__(128) unsigned char dyn[];
-    __shared__ SkShared sh;
-    uint64_t* full = reinterpret_cast<uint64_t*>(dyn);
-    uint64_t* empty = full + MAX_STAGES;
-    float* ring = reinterpret_cast<float*>(dyn + S.off_ring);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const SolveParams& P0 = M.P[0];
-    int64_t r0, r1;
-    cta_rows(P0.I, S.rows_per_stage, P0.V, blockIdx.x, gridDim.x, &r0, &r1);
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < S.stages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], NCW);
-        }
-        sh.s_stop = 0;
-        sh.s_bad = 0;
-        sh.s_dec = 0;
-        mbar_fence_init();
-    }
-    __syncthreads();
-    if (warp == NCW) {
-        if (lane == 0)
-            stream_rows_producer(P0.C, P0.ld, r0, r1, S, ring, full, empty, &sh.s_stop, &M.grp->status, P0.spin);
-        return;
-    }
-    GroupCtx g{(int)gridDim.x, (int)blockIdx.x, &M.grp->bar, 0u, &M.grp->status, &M.grp->status};
-    ms_consumers<TW, VPT, NS, RC>(M, S, g, &sh, dyn, r0, r1);
-}
 
 // The launch's status into every solve's loop state (the finalize kernels read it there).
 __global__ void sk_multi_status(const LoopState* grp, LoopState* a, LoopState* b, LoopState* c) {
@@ -217,38 +127,6 @@ __global__ void sk_summary(const double* __restrict__ epart, int nb, const doubl
 // Host side.
 // ------------------------------------------------------------------------------------------
 namespace {
-
-struct Kernels {
-    const void* solve;
-    int tw, vpt, ncw;
-    int nthreads;  // block size: the consumer warps, plus the producer warp where C is streamed
-};
-
-template <int TW, int VPT, bool EUC>
-Kernels kernels_for() {
-    if constexpr (EUC) return Kernels{(const void*)sk_solve_euclid<TW, VPT>, TW, VPT, Cons<TW>::NCW, Cons<TW>::NCW * 32};
-    else return Kernels{(const void*)sk_solve<TW, VPT>, TW, VPT, Cons<TW>::NCW, Cons<TW>::NT};
-}
-
-// One-warp teams (TW = 1) get VPT = ceil(J4 / 32) exactly; chunk_inside() relies on it.
-template <bool EUC>
-bool pick_kernels_t(int J, Kernels* k) {
-    const int J4 = (J + 3) / 4;
-    if (J4 <= 32) *k = kernels_for<1, 1, EUC>();
-    else if (J4 <= 64) *k = kernels_for<1, 2, EUC>();
-    else if (J4 <= 96) *k = kernels_for<1, 3, EUC>();
-    else if (J4 <= 128) *k = kernels_for<1, 4, EUC>();
-    else if (J4 <= 160) *k = kernels_for<1, 5, EUC>();
-    else if (J4 <= 192) *k = kernels_for<1, 6, EUC>();
-    else if (J4 <= 224) *k = kernels_for<1, 7, EUC>();
-    else if (J4 <= 256) *k = kernels_for<1, 8, EUC>();
-    else if (J4 <= 512) *k = kernels_for<2, 8, EUC>();
-    else if (J4 <= 1024) *k = kernels_for<4, 8, EUC>();
-    else if (J4 <= 2048) *k = kernels_for<8, 8, EUC>();
-    else return false;
-    return true;
-}
-bool pick_kernels(int J, Kernels* k) { return pick_kernels_t<false>(J, k); }
 
 // Stage geometry, shared-memory layout and grid of the persistent kernel: one CTA per row
 // partition (at most one per SM).
@@ -458,7 +336,7 @@ ot_status enqueue_solve_f32(ot_assoc_ctx* ctx, const SolveArgs& a, SolveSummary*
     const int Jp = (int)round_up(J, 4);
     Kernels kk;
     const bool euc = a.dev_xy != nullptr;
-    if (!(euc ? pick_kernels_t<true>(J, &kk) : pick_kernels(J, &kk)))
+    if (!(euc ? pick_euclid(J, &kk) : pick_kernels(J, &kk)))
         return set_error(ctx, OT_EUNSUPPORTED, "J=%d above 8192", J);
     LoopLaunch LL;
     st = plan_solve(kk, I, Jp, a.ld, ctx->num_sms, 1 << 30, &LL);
@@ -473,31 +351,6 @@ ot_status enqueue_solve_f32(ot_assoc_ctx* ctx, const SolveArgs& a, SolveSummary*
     e = cudaMemcpyAsync(dest, B.summ, sizeof(SolveSummary), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "summary copy");
     return OT_OK;
-}
-
-// Kernels of the multi-solve launch.  Up to 128 float4 chunks a row, one-warp teams keep
-// three solves' accumulators with the row (4 chunks a lane).  Wider rows: two solves on
-// one-warp teams with the cell values computed twice (the row stays with the one-warp
-// team of a single solve), three solves on wider teams (4 chunks a lane).
-template <int TW, int VPT, int NS, bool RC>
-Kernels multi_for() {
-    return Kernels{(const void*)sk_solve_multi<TW, VPT, NS, RC>, TW, VPT, Cons<TW>::NCW, Cons<TW>::NT};
-}
-bool pick_multi(int J, int n, Kernels* k) {
-    const int J4 = (J + 3) / 4;
-    if (J4 <= 32) *k = multi_for<1, 1, 3, false>();
-    else if (J4 <= 64) *k = multi_for<1, 2, 3, false>();
-    else if (J4 <= 96) *k = multi_for<1, 3, 3, false>();
-    else if (J4 <= 128) *k = multi_for<1, 4, 3, false>();
-    else if (n <= 2 && J4 <= 160) *k = multi_for<1, 5, 2, true>();
-    else if (n <= 2 && J4 <= 192) *k = multi_for<1, 6, 2, true>();
-    else if (n <= 2 && J4 <= 224) *k = multi_for<1, 7, 2, true>();
-    else if (n <= 2 && J4 <= 256) *k = multi_for<1, 8, 2, true>();
-    else if (J4 <= 256) *k = multi_for<2, 4, 3, false>();
-    else if (J4 <= 512) *k = multi_for<4, 4, 3, false>();
-    else if (J4 <= 1024) *k = multi_for<8, 4, 3, false>();
-    else return false;
-    return true;
 }
 
 ot_status launch_solve_f32(ot_assoc_ctx* ctx, const SolveArgs& a, SolveSummary* sum_host) {

@@ -165,12 +165,12 @@ __device__ __forceinline__ float log2_corr(float r) {
     return fabsf(u) < 0.0078125f ? series : sfu;
 }
 
-// A lane's chunk v is certainly inside the row when the dispatch chose VPT = ceil(J4 / 32)
-// for a one-warp team (pick_kernels does exactly that for TW = 1): then every chunk but the
-// lane's last ends at or before column J.  Wider teams check every chunk.
+// A lane's chunk v is certainly inside the row when the dispatch chose VPT = ceil(J4 / (32 TW))
+// (pick_kernels and the batched forms do; the multi-solve's wide teams, VPT = 4, do not): then
+// every chunk but the lane's last ends at or before column J.
 template <int TW, int VPT>
 __device__ __forceinline__ constexpr bool chunk_inside(int v) {
-    return TW == 1 && v < VPT - 1;
+    return (TW == 1 || VPT > 4) && v < VPT - 1;
 }
 
 // Row load from a shared-memory stage; chunks that can leave the row are checked.
@@ -392,6 +392,18 @@ inline bool plan_stage(int nteams, int64_t I, int Jp, int64_t ld, int nb, int st
     return true;
 }
 
+// A consumer's place in the ring of stages: the stage and the parity of its current use.
+struct RingPos {
+    int st = 0;
+    uint32_t ph = 0;
+    __device__ __forceinline__ void next(int stages) {
+        if (++st == stages) {
+            st = 0;
+            ph ^= 1u;
+        }
+    }
+};
+
 // Sum of (s, e) pairs over a warp with error-free additions.
 __device__ __forceinline__ void warp_sum_pair(float& s, float& e) {
 #pragma unroll
@@ -412,6 +424,7 @@ struct SkShared {
     double sh_sum[24][2];   // per-warp setup sums (up to 24 consumer warps)
     int s_dec, s_ok, s_bad;
     volatile int s_stop;    // consumers -> producer: stop streaming
+    uint32_t tmem;          // tensor-memory address of the column potentials (see G_to_tmem)
     int pend[VMAX + 1];     // stage blocks (from the CTA's first row) at which its partitions end
 };
 
@@ -500,7 +513,7 @@ static constexpr int FIN_ROWS = 16;
 template <int TW, int VPT, bool EUC = false>
 __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const StreamCfg& S, SkShared* sh,
                                                   unsigned char* dyn, int64_t r0, int nrow, int v0, int v1,
-                                                  const float2* Fold, uint32_t& cseq, int* abort) {
+                                                  const float2* Fold, RingPos& pos, int* abort) {
     constexpr int NCW = Cons<TW>::NCW;
     constexpr int TT = 32 * TW, NTEAMS = NCW / TW, NC = NCW * 32;
     uint64_t* full = reinterpret_cast<uint64_t*>(dyn);
@@ -537,8 +550,8 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
     int vp = v0, vbeg = 0;
     int vend = v0 < v1 ? pend[v0] : 0;
     for (int kb = 0; kb < nblk; ++kb) {
-        const int st = (int)(cseq % (uint32_t)S.stages);
-        const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
+        const int st = pos.st;
+        const uint32_t ph = pos.ph;
         const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, abort);
         const int lr0 = kb * rs_;
         const int rows = min(rs_, nrow - lr0);
@@ -590,7 +603,7 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
         }
         __syncwarp();
         if (!EUC && lane == 0) mbar_arrive(&empty[st]);
-        ++cseq;
+        pos.next(S.stages);
         const bool at_end = (kb + 1 == vend);
         if ((kb + 1 - vbeg) % every == 0 || at_end) {
             if (defer) {
@@ -645,6 +658,223 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
             const float2 F = Fold[r];
             P.f_nat[r0 + r] = P.eps_ln2 * ((double)F.x + (double)F.y + log2((double)__ldg(P.p + r0 + r)));
         }
+}
+
+// ---- packed FP32 pairs: one instruction for two columns (fma/add .f32x2), each half rounded
+// exactly as the scalar operation rounds it. ------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Sums of R rows' per-lane values over the team, each in the order of team_reduce; every lane
+// gets all R.  Two rows share one butterfly: after the first exchange the lower half-warp
+// holds row 0's sums and the upper half row 1's (the same pairs are added), so two rows take
+// the shuffles of one plus one exchange, and wider teams one named barrier.
+template <int TW, int R>
+__device__ __forceinline__ void team_sum_rows(float (&v)[R], float* red, int nteams, const Team<TW>& tm, int& par) {
+    if constexpr (R == 1) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        if constexpr (TW > 1) {  // a team's slots are the same ones as for two rows
+            float* r = red + (par * nteams + tm.team) * (2 * TW);
+            if (tm.lane == 0) r[tm.wit] = v[0];
+            bar_named(1 + tm.team, 32 * TW);
+            float a = r[0];
+#pragma unroll
+            for (int w = 1; w < TW; ++w) a += r[w];
+            v[0] = a;
+            par ^= 1;
+        }
+    } else {
+        static_assert(R == 2, "one or two rows");
+        const bool up = tm.lane >= 16;
+        float s = (up ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if constexpr (TW == 1) {
+            const float w = __shfl_xor_sync(0xffffffffu, s, 16);
+            v[0] = up ? w : s;
+            v[1] = up ? s : w;
+        } else {
+            float* r = red + (par * nteams + tm.team) * (2 * TW);
+            if ((tm.lane & 15) == 0) r[(up ? TW : 0) + tm.wit] = s;
+            bar_named(1 + tm.team, 32 * TW);
+            float a = r[0], b = r[TW];
+#pragma unroll
+            for (int w = 1; w < TW; ++w) {
+                a += r[w];
+                b += r[TW + w];
+            }
+            v[0] = a;
+            v[1] = b;
+            par ^= 1;
+        }
+    }
+}
+
+// Column potentials in tensor memory: the eight words of chunk v (four high parts, four low
+// parts) of a lane at columns 8 v .. 8 v + 7 of its warp's quarter.  Lane positions repeat
+// every TW warps, so one copy per quarter serves every warp of the CTA (two for teams of 8).
+// The sweep reads G (eight bytes a column) once per row: from shared memory that was two thirds
+// of its shared-memory wavefronts (84 a row of 800 columns, with 25 more for the copy that
+// fills the ring), the busiest unit of the sweep.  Out of tensor memory the sweep of a
+// 50,000 x 800 solve takes 41,000 cycles a CTA instead of 46,600, and the whole solve 0.98 ms
+// instead of 1.00 (1.04 before the packed arithmetic); 100,000 x 1,536: 2.50 ms against 3.03.
+template <int TW, int VPT>
+constexpr int tmem_cols() {
+    constexpr int n = 8 * VPT * (TW == 8 ? 2 : 1);
+    return n <= 32 ? 32 : (n <= 64 ? 64 : 128);
+}
+template <int TW, int VPT>
+__device__ __forceinline__ uint32_t tmem_G(uint32_t base, const Team<TW>& tm) {
+    const uint32_t warp = threadIdx.x >> 5;
+    return base + ((warp & 3u) << 21) + (TW == 8 ? (uint32_t)(tm.wit >> 2) * (8 * VPT) : 0u);
+}
+// Copy G from shared memory to tensor memory (all consumer warps call; G complete in Gs before,
+// visible to every consumer warp after).
+template <int TW, int VPT>
+__device__ __forceinline__ void G_to_tmem(uint32_t base, const float* Gs, int Jp, const Team<TW>& tm) {
+    constexpr int WRITERS = TW == 8 ? 8 : 4, TT = 32 * TW;
+    if ((threadIdx.x >> 5) < WRITERS) {
+        const uint32_t a = tmem_G<TW, VPT>(base, tm);
+        tmem_fence_after();
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            const int col = 4 * (tm.tl + TT * v);
+            float4 hi = make_float4(0.f, 0.f, 0.f, 0.f), lo = hi;
+            if (col < Jp) {
+                hi = *reinterpret_cast<const float4*>(Gs + col);
+                lo = *reinterpret_cast<const float4*>(Gs + Jp + col);
+            }
+            __syncwarp();
+            tmem_st8(a + 8 * v, hi, lo);
+        }
+        tmem_wait_st();
+        tmem_fence_before();
+    }
+    bar_named(CONS_BAR, Cons<TW>::NCW * 32);
+    tmem_fence_after();
+}
+
+// Rows a team takes at once.  Two rows of up to 6 chunks a lane fit the registers (128 a
+// thread); at 7 chunks the second row spills (50,000 x 800: 1.01 ms with two rows, 0.98 with
+// one).  Wider teams stay at one: their rows come from HBM, not L2, at the sizes that matter,
+// and two rows took 2.55 ms against 2.50 on 100,000 x 1,536.  1000 x 50 takes 245 us with two
+// rows, 255 with one.
+template <int TW, int VPT, bool EUC>
+__host__ __device__ constexpr int rows_per_pass() {
+    return EUC || TW > 1 || VPT > 6 ? 1 : 2;
+}
+
+// One plan-scale pass of a team over R rows of C at once (row[k]: the staged row, or unused
+// when EUC with the device at dxy[k]): t_ij = 2^(F'_i + G_j - k C_ij), the row sums r_i, the
+// row update and residual, and the column accumulators acc += t p^ / r, row 0 before row 1.
+// Bound by instruction issue and by the latency of a row's chain (shared-memory loads, ex2,
+// the team sum, the update) once C streams: two rows in flight hide one chain behind the
+// other and share the loads of G, and packed arithmetic halves the instructions of the
+// exponent and the accumulation (50,000 x 800: 1.04 -> 1.00 ms, 100,000 x 1,536: 3.98 -> 3.03,
+// with the chunk count of a lane fitted to the row for wide teams too).  Every operation
+// rounds as for one row at a time, so results are the same bit for bit.
+template <int TW, int VPT, bool EUC, int R>
+__device__ __forceinline__ void sweep_rows(const float* const (&row)[R], const float2 (&dxy)[R], uint32_t tG, int J,
+                                           int Jp, const float* rxs, f32x2 nk_hi, f32x2 nk_lo, const float2* Fold,
+                                           float2* Fnew, const float* Ps, const int (&lr)[R], float* red, int nteams,
+                                           const Team<TW>& tm, int& par, f32x2 (&acc)[VPT][2], float& errt) {
+    constexpr int TT = 32 * TW;
+    __syncwarp();
+    f32x2 t[R][VPT][2], Fh[R], Fl[R];
+    float2 F[R];
+    float rsum[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        F[k] = Fold[lr[k]];
+        Fh[k] = pack2(F[k].x, F[k].x);
+        Fl[k] = pack2(F[k].y, F[k].y);
+        rsum[k] = 0.f;
+    }
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+        // lanes past the row (last chunk only) take column 0 and drop what they get: no branch,
+        // so the warp stays converged for the tensor-memory loads
+        const bool all_in = chunk_inside<TW, VPT>(v);
+        const int at = 4 * (tm.tl + TT * v);
+        const int col = all_in || at < J ? at : 0;
+        float4 g4, l4;
+        tmem_ld8(tG + 8 * v, g4, l4);
+        const f32x2 gh[2] = {pack2(g4.x, g4.y), pack2(g4.z, g4.w)}, gl[2] = {pack2(l4.x, l4.y), pack2(l4.z, l4.w)};
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            f32x2 c[2];
+            if constexpr (EUC) {
+                const float4 e = euclid_chunk(dxy[k], rxs, rxs + Jp, col, J);
+                c[0] = pack2(e.x, e.y);
+                c[1] = pack2(e.z, e.w);
+            } else {
+                const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(row[k] + col);
+                c[0] = e.x;
+                c[1] = e.y;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // the exponent of expo2, two columns at a time
+                const float2 x = unpack2(
+                    add2(add2(fma2(c[h], nk_hi, Fh[k]), gh[h]), fma2(c[h], nk_lo, add2(Fl[k], gl[h]))));
+                float t0 = ex2(x.x), t1 = ex2(x.y);
+                if (!all_in) {
+                    t0 = at + 2 * h < J ? t0 : 0.f;
+                    t1 = at + 2 * h + 1 < J ? t1 : 0.f;
+                }
+                rsum[k] += t0;
+                rsum[k] += t1;
+                t[k][v][h] = pack2(t0, t1);
+            }
+        }
+    }
+    team_sum_rows<TW, R>(rsum, red, nteams, tm, par);
+    float d[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const float ph = Ps[lr[k]];
+        errt = fmaf(ph, fabsf(rsum[k] - 1.0f), errt);
+        d[k] = __fdividef(ph, rsum[k]);
+    }
+    if constexpr (R == 1) {
+        // every lane forms the update (no divergent branch); one lane stores it
+        const float2 Fn = df_sub(F[0], log2_corr(rsum[0]));
+        if (tm.tl == 0) Fnew[lr[0]] = Fn;
+    } else {  // the lower half-warp forms row 0's update, the upper row 1's
+        const bool up = tm.lane >= 16;
+        const float2 Fu = up ? F[1] : F[0];
+        const float2 Fn = df_sub(Fu, log2_corr(up ? rsum[1] : rsum[0]));
+        if ((tm.lane & 15) == 0 && tm.wit == 0) Fnew[up ? lr[1] : lr[0]] = Fn;
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const f32x2 dk = pack2(d[k], d[k]);
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            acc[v][0] = fma2(t[k][v][0], dk, acc[v][0]);
+            acc[v][1] = fma2(t[k][v][1], dk, acc[v][1]);
+        }
+    }
 }
 
 // The consumer warps' part of one solve (Algorithm 1 on the CTA's partitions, rows [r0, r1)):
@@ -800,13 +1030,13 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         bar_named(CONS_BAR, NC);
     }
     const Team<TW> tm;
-    uint32_t cseq = 0;
+    RingPos pos;
     if (P.F_in) {  // finalize only
         for (int r = tid; r < nrow; r += NC) Fs[r] = P.F_in[r0 + r];
         load_G_smem(P.G_in, J, Jp, Gs, tid, NC);
         bar_named(CONS_BAR, NC);
         *ret_par = 0;
-        sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fs, cseq, g.abort);
+        sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fs, pos, g.abort);
         if (tid == 0) s_stop = 1;
         return true;
     }
@@ -831,8 +1061,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         for (int vp = v0; vp < v1; ++vp) {
             const int vend = pend[vp];
             for (; kb < vend; ++kb) {
-                const int st = (int)(cseq % (uint32_t)S.stages);
-                const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
+                const int st = pos.st;
+                const uint32_t ph = pos.ph;
                 const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
                 const int lr0 = kb * rs_;
                 const int rows = min(rs_, nrow - lr0);
@@ -885,7 +1115,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 }
                 __syncwarp();
                 if (!EUC && lane == 0) mbar_arrive(&empty[st]);
-                ++cseq;
+                pos.next(S.stages);
             }
             float* cp = P.colpart + (int64_t)vp * Jp;
             cta_col_sum<TW, VPT>(comb, acc, J, Jp, tm, [&](int j, float sum) { cp[j] = sum; });
@@ -931,8 +1161,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         for (int vp = v0; vp < v1; ++vp) {
           const int vend = pend[vp];
           for (; kb < vend; ++kb) {
-            const int st = (int)(cseq % (uint32_t)S.stages);
-            const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
+            const int st = pos.st;
+            const uint32_t ph = pos.ph;
             const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
             const int lr0 = kb * rs_;
             const int rows = min(rs_, nrow - lr0);
@@ -994,7 +1224,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             }
             __syncwarp();
             if (!EUC && lane == 0) mbar_arrive(&empty[st]);
-            ++cseq;
+            pos.next(S.stages);
           }
             // end of partition vp: merge the teams' (max, sum) pairs in two rounds through
             // the float buffer, the column maxima first (held in Gs meanwhile), then the sums
@@ -1117,76 +1347,79 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     // Each partition adds its column partials (and row residual) as fixed-point integers into
     // the row of totals of this sweep; after the one grid barrier of the iteration every CTA
     // reads the totals and forms all column updates itself in its shared-memory copy of G.
+    constexpr int RPP = rows_per_pass<TW, VPT, EUC>();
+    // a team's rows of a block come in pairs when there is an even number of them; otherwise a
+    // step takes two blocks, if the ring has stages to spare for that
+    const int step_blocks = RPP == 2 && (S.rpt & 1) && S.stages >= 4 ? 2 : 1;
+    const uint32_t tG = tmem_G<TW, VPT>(sh->tmem, tm);
+    G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
+    const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
     for (int s = 2;; ++s) {
         unsigned long long* acc_s = ACC + (size_t)(s % 3) * (Jp + 4);
         const float2* Fold = Fs + ((s - 1) & 1) * S.rmax;  // F'^(s-1)
         float2* Fnew = Fs + (s & 1) * S.rmax;
-        float4 acc[VPT];
+        f32x2 acc[VPT][2];
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
         float errt = 0.f;  // every lane of a team holds the same value
         int kb = 0;
         for (int vp = v0; vp < v1; ++vp) {
           const int vend = pend[vp];
-          for (; kb < vend; ++kb) {
-            const int st = (int)(cseq % (uint32_t)S.stages);
-            const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
-            const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
-            const int lr0 = kb * rs_;
-            const int rows = min(rs_, nrow - lr0);
-            const float* stage = ring + (size_t)st * S.stage_floats;
-            for (int j = 0; ok && j < S.rpt; ++j) {
-                const int rr = tm.team + NTEAMS * j;
-                if (rr >= rows) break;
-                const int lr = lr0 + rr;
-                float4 x[VPT];
-                if constexpr (EUC)
-                    euclid_row<TW, VPT>(__ldg(P.dev_xy + r0 + lr), rxs, rxs + Jp, J, tm.tl, x);
-                else
-                    load_row_smem<TW, VPT>(stage + (size_t)rr * P.ld, J, tm.tl, x);
-                const float2 F = Fold[lr];
-                float rsum = 0.f;
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    const int col = 4 * (tm.tl + TT * v);
-                    if (chunk_inside<TW, VPT>(v) || col < J) {  // chunks past the row carry no mass
-                        float4 gv = *reinterpret_cast<const float4*>(Gs + col);
-                        float4 gl = *reinterpret_cast<const float4*>(Gs + Jp + col);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float t = ex2(expo2(F.x, F.y + comp(gl, c), comp(gv, c), comp(x[v], c), P.k_hi, P.k_lo));
-                            comp(x[v], c) = t;
-                            rsum += t;
-                        }
-                    } else {
-                        x[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+          while (kb < vend) {
+            // a step: one stage block, or two when a team's rows in a block do not pair up
+            const int nblk = min(step_blocks, vend - kb);
+            const RingPos p0 = pos;
+            bool ok = EUC || mbar_try_wait(&full[p0.st], p0.ph) || mbar_wait_bounded(&full[p0.st], p0.ph, P.spin, g.abort);
+            pos.next(S.stages);
+            RingPos p1 = pos;
+            if (nblk == 2) {
+                ok = ok && (EUC || mbar_try_wait(&full[p1.st], p1.ph) ||
+                            mbar_wait_bounded(&full[p1.st], p1.ph, P.spin, g.abort));
+                pos.next(S.stages);
+            }
+            const float* stage0 = ring + (size_t)p0.st * S.stage_floats + (size_t)tm.team * P.ld;
+            const float* stage1 = ring + (size_t)p1.st * S.stage_floats + (size_t)tm.team * P.ld;
+            const int lr0 = kb * rs_ + tm.team;  // the team's rows are lr0 + NTEAMS q
+            const int nq = ok ? min(nblk * S.rpt, (nrow - lr0 + NTEAMS - 1) / NTEAMS) : 0;
+            auto staged = [&](int q) {
+                return q < S.rpt ? stage0 + (size_t)(NTEAMS * q) * P.ld : stage1 + (size_t)(NTEAMS * (q - S.rpt)) * P.ld;
+            };
+            for (int q = 0; q < nq; q += RPP) {
+                if constexpr (RPP == 2) {
+                    if (q + 1 < nq) {
+                        const int lr[2] = {lr0 + NTEAMS * q, lr0 + NTEAMS * (q + 1)};
+                        const float* const row[2] = {staged(q), staged(q + 1)};
+                        const float2 dxy[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                        sweep_rows<TW, VPT, EUC, 2>(row, dxy, tG, J, Jp, rxs, nk_hi, nk_lo, Fold, Fnew, Ps, lr, red, NTEAMS,
+                                                    tm, par, acc, errt);
+                        continue;
                     }
                 }
-                rsum = team_reduce<TW, float, false>(rsum, red, NTEAMS, tm, par);
-                const float ph = Ps[lr];
-                // every lane forms the update (no divergent branch); one lane stores it
-                const float2 Fn = df_sub(F, log2_corr(rsum));
-                if (tm.tl == 0) Fnew[lr] = Fn;
-                errt = fmaf(ph, fabsf(rsum - 1.0f), errt);
-                const float d = __fdividef(ph, rsum);
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    acc[v].x = fmaf(x[v].x, d, acc[v].x);
-                    acc[v].y = fmaf(x[v].y, d, acc[v].y);
-                    acc[v].z = fmaf(x[v].z, d, acc[v].z);
-                    acc[v].w = fmaf(x[v].w, d, acc[v].w);
-                }
+                const int lr[1] = {lr0 + NTEAMS * q};
+                const float* const row[1] = {staged(q)};
+                const float2 dxy[1] = {EUC ? __ldg(P.dev_xy + r0 + lr[0]) : make_float2(0.f, 0.f)};
+                sweep_rows<TW, VPT, EUC, 1>(row, dxy, tG, J, Jp, rxs, nk_hi, nk_lo, Fold, Fnew, Ps, lr, red, NTEAMS, tm,
+                                            par, acc, errt);
             }
             __syncwarp();
-            if (!EUC && lane == 0) mbar_arrive(&empty[st]);
-            ++cseq;
+            if (!EUC && lane == 0) {
+                mbar_arrive(&empty[p0.st]);
+                if (nblk == 2) mbar_arrive(&empty[p1.st]);
+            }
+            kb += nblk;
           }
             // end of partition vp: its column partials (teams in order) and row residual.  The
             // FP32 partial is kept for the exact path and added to the column's total as
             // round(partial 2^S_j); a partial too large for the total marks the column.
             if (tm.tl == 0) errf[tm.team] = errt;
             float* cp = P.colpart + (int64_t)vp * Jp;
-            cta_col_sum<TW, VPT>(comb, acc, J, Jp, tm, [&](int j, float sum) {
+            float4 part[VPT];
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                const float2 a = unpack2(acc[v][0]), b = unpack2(acc[v][1]);
+                part[v] = make_float4(a.x, a.y, b.x, b.y);
+            }
+            cta_col_sum<TW, VPT>(comb, part, J, Jp, tm, [&](int j, float sum) {
                 cp[j] = sum;
                 const int sx = SX[j];
                 const float x = ldexpf(sum, sx);
@@ -1200,10 +1433,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 s_bad = 0;
             }
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
             errt = 0.f;
             if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // errf is read by thread 0 above
         }
+        tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
         // the constant per-column values of this thread's first round of column updates are
         // loaded before the barrier, so only the totals cross L2 after it
         constexpr int CU = 3;
@@ -1228,7 +1462,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             if (P.F_out)
                 for (int r = tid; r < nrow; r += NC) P.F_out[r0 + r] = Fold[r];
             *ret_par = (s - 1) & 1;
-            if (P.fpart) sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fold, cseq, g.abort);
+            if (P.fpart) sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
             if (tid == 0) s_stop = 1;
             return true;
         }
@@ -1288,6 +1522,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 if (tid == 0) s_stop = 1;
                 return false;
             }
+            G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
         }
     }
 #undef OTA_BARRIER_CHECK

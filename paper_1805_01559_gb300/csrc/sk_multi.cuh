@@ -76,7 +76,7 @@ inline bool plan_multi(int nteams, int n, int64_t I, int Jp, int64_t ld, int nb,
 template <int TW, int VPT>
 __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const StreamCfg& S, GroupCtx& g, SkShared* sh,
                                                unsigned char* dyn, float* Gs, float2* F1, const float* Ps,
-                                               int nrow, int v0, int v1, uint32_t& cseq, int& par) {
+                                               int nrow, int v0, int v1, RingPos& pos, int& par) {
     constexpr int NCW = Cons<TW>::NCW;
     constexpr int TT = 32 * TW, NTEAMS = NCW / TW, NC = NCW * 32;
     constexpr int HALF = (NTEAMS + 1) / 2;
@@ -101,8 +101,8 @@ __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const Strea
     for (int vp = v0; vp < v1; ++vp) {
         const int vend = pend[vp];
         for (; kb < vend; ++kb) {
-            const int st = (int)(cseq % (uint32_t)S.stages);
-            const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
+            const int st = pos.st;
+            const uint32_t ph = pos.ph;
             const bool ok = mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
             const int lr0 = kb * rs_;
             const int rows = min(rs_, nrow - lr0);
@@ -156,7 +156,7 @@ __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const Strea
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[st]);
-            ++cseq;
+            pos.next(S.stages);
         }
         // end of partition vp: teams' (max, sum) pairs merged in team order
         for (int round = 0; round < 2; ++round) {
@@ -394,13 +394,13 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
     }
     // LQ of solve s is read after the first grid barrier of its first iteration
     const Team<TW> tm;
-    uint32_t cseq = 0;
+    RingPos pos;
     int par = 0;
 
     // ---- the exact first iteration, one solve after the other ---------------------------
     for (int s = 0; s < n; ++s) {
         if (!ms_first_sweep<TW, VPT>(M.P[s], S, g, sh, dyn, Gbase + (size_t)2 * s * Jp,
-                                      Fbase + (size_t)s * 2 * S.rmax + S.rmax, Ps, nrow, v0, v1, cseq, par)) {
+                                      Fbase + (size_t)s * 2 * S.rmax + S.rmax, Ps, nrow, v0, v1, pos, par)) {
             if (tid == 0) s_stop = 1;
             return false;
         }
@@ -422,8 +422,8 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
         for (int vp = v0; vp < v1; ++vp) {
             const int vend = pend[vp];
             for (; kb < vend; ++kb) {
-                const int st = (int)(cseq % (uint32_t)S.stages);
-                const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
+                const int st = pos.st;
+                const uint32_t ph = pos.ph;
                 const bool ok = mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P0.spin, g.abort);
                 const int lr0 = kb * rs_;
                 const int rows = min(rs_, nrow - lr0);
@@ -535,7 +535,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[st]);
-                ++cseq;
+                pos.next(S.stages);
             }
             // end of partition vp: each active solve's column partials and row residual
 #pragma unroll
@@ -629,7 +629,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
         StreamCfg Ss = S;
         Ss.off_G = S.off_G + (int)(sizeof(float) * (size_t)2 * s * Jp);
         const float2* Fold = Fbase + (size_t)s * 2 * S.rmax + retp[s] * S.rmax;
-        sk_finalize_sweep<TW, VPT>(M.P[s], Ss, sh, dyn, r0, nrow, v0, v1, Fold, cseq, g.abort);
+        sk_finalize_sweep<TW, VPT>(M.P[s], Ss, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
         bar_named(CONS_BAR, NC);
     }
     if (tid == 0) s_stop = 1;

@@ -1,0 +1,49 @@
+"""The plan-scale sweeps at the edges of their tiles: every width at which a lane takes another
+chunk or a row a wider team, and row counts that leave a team one row, an odd row, or none.
+
+Tolerance: that of the fixed-iteration tests of test_gpu_parity.py (a plan entry within 2e-5
+relative plus 1e-12 of the mass after 3 iterations; derived there from the rounding of the
+exponent, ex2.approx and FP32 sums of up to 8192 terms, which these sweeps share).
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1805_01559_gb300 import binding
+    c = binding.Context(0)
+    yield c
+    c.close()
+
+
+WIDTHS = [1, 3, 4, 127, 128, 129, 385, 512, 640, 641, 768, 769, 896, 897, 1024, 1025, 1280, 1281, 1535, 1537, 1793,
+          2048, 2049, 2561, 3073, 3585, 4096, 4097, 5121, 6145, 7169, 8192]
+SHAPES = ([(I, J) for J in WIDTHS for I in (67,)]
+          + [(I, J) for J in (50, 300, 650, 1300) for I in (1, 14, 16, 31, 46, 105, 211, 700)])
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_sweep_tile_edges(ctx, shape):
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 10007 + J))
+    C = rng.uniform(0.0, 1.0, (I, J)).astype(np.float32)
+    p = rng.lognormal(0.0, 1.0, I)
+    q = rng.uniform(0.5, 1.5, J)
+    p, q = (p / p.sum()).astype(np.float32), (q / q.sum()).astype(np.float32)
+    pad = torch.full((I, (J + 3) // 4 * 4), float("nan"), dtype=torch.float32, device="cuda")  # padding is never read as mass
+    pad[:, :J] = torch.from_numpy(C).cuda()
+    res = ctx.solve_cost(pad[:, :J], torch.from_numpy(p).cuda(), torch.from_numpy(q).cuda(), 0.1, tol=0.0, max_iter=3,
+                         want_pi=True)
+    C64 = C.astype(np.float64)
+    f, g, _, _ = oracle.sinkhorn(C64, p, q, 0.1, 0.0, 3)
+    pi = oracle.plan(C64, f, g, 0.1)
+    err = np.abs(res.pi.cpu().numpy().astype(np.float64) - pi)
+    assert (err <= 2e-5 * pi + 1e-12).all(), float((err / pi).max())
