@@ -97,21 +97,30 @@ __device__ __forceinline__ bool bt_finalize(const BInst& D, const SolveParams& P
         }
     }
     if (!group_sync(gbar, gsize, s_gen, abort, spin)) return false;
-    if (rank == 0 && threadIdx.x == 0) {
+    // Totals by one warp: its lanes stride the group's gsize x BT_NW warp partials, then one
+    // FP64 tree.  (One thread walking them cost a group of 152 CTAs, 2,432 entries, about
+    // 180 us a solve: ten warm steps on a 20,000 x 400 cell took 3.5 ms, 1.71 with this.)
+    if (rank == 0 && warp == 0) {
         const double* rowerr = grp.fred + (size_t)gsize * BT_NW * 2;
         double ec = 0.0, co = 0.0, er = 0.0;
-        for (int k = 0; k < gsize * BT_NW; ++k) {
-            ec += grp.fred[2 * k];
-            co += grp.fred[2 * k + 1];
+        for (int k = lane; k < gsize * BT_NW; k += 32) {
+            const double2 v = __ldcg(reinterpret_cast<const double2*>(grp.fred) + k);
+            ec += v.x;
+            co += v.y;
         }
-        for (int k = 0; k < P.V; ++k) er += rowerr[k];
-        out->cost = co * P.sc->sp;
-        out->err_row = er;
-        out->err_col = ec;
-        out->err_loop = grp.ls->err;
-        out->iters = grp.ls->iters;
-        out->converged = grp.ls->converged;
-        out->done = 1;  // out->status holds whatever the solve reported (DEV_OK normally)
+        for (int k = lane; k < P.V; k += 32) er += __ldcg(rowerr + k);
+        ec = warp_sum(ec);
+        co = warp_sum(co);
+        er = warp_sum(er);
+        if (lane == 0) {
+            out->cost = co * P.sc->sp;
+            out->err_row = er;
+            out->err_col = ec;
+            out->err_loop = grp.ls->err;
+            out->iters = grp.ls->iters;
+            out->converged = grp.ls->converged;
+            out->done = 1;  // out->status holds whatever the solve reported (DEV_OK normally)
+        }
     }
     return true;
 }
