@@ -47,3 +47,25 @@ def test_sweep_tile_edges(ctx, shape):
     pi = oracle.plan(C64, f, g, 0.1)
     err = np.abs(res.pi.cpu().numpy().astype(np.float64) - pi)
     assert (err <= 2e-5 * pi + 1e-12).all(), float((err / pi).max())
+
+
+# Row counts around a tile's 8 rows, and widths around those at which a tile takes fewer rows.
+@pytest.mark.parametrize("shape", [(1, 3), (7, 64), (8, 65), (9, 31), (1217, 20), (40, 2880), (40, 2881), (21, 4817),
+                                   (13, 7200), (11, 8192)])
+def test_fp64_tile_edges(ctx, shape):
+    """FP64 form against the oracle after 4 iterations: both in doubles, a few ulp an iteration
+    on exponents of up to 20, so 1e-10 relative as in test_gpu_f64.py."""
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 10007 + J))
+    C = rng.uniform(0.0, 1.0, (I, J))
+    p = rng.lognormal(0.0, 1.0, I)
+    q = rng.uniform(0.5, 1.5, J)
+    q *= p.sum() / q.sum()
+    res = ctx.solve_f64(torch.from_numpy(C).cuda(), torch.from_numpy(p).cuda(), torch.from_numpy(q).cuda(), 0.05, tol=0.0,
+                        max_iter=4)
+    f, g, _, _ = oracle.sinkhorn(C, p, q, 0.05, 0.0, res.iters)
+    np.testing.assert_allclose(oracle.plan(C, res.f.cpu().numpy(), res.g.cpu().numpy(), 0.05), oracle.plan(C, f, g, 0.05),
+                               rtol=1e-10, atol=1e-300)
+    cost, rho, _, _ = oracle.finalize(C, f, g, p, q, 0.05)
+    assert res.transport_cost == pytest.approx(cost, rel=1e-12)
+    np.testing.assert_allclose(res.rrh_load.cpu().numpy(), rho, rtol=1e-12)
