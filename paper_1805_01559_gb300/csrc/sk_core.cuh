@@ -42,13 +42,22 @@ struct LoopState {
 //   [2 Jp, 3 Jp)    log2 q^_j (FP64)
 //   [3 Jp, 4 Jp)    log2 q^_j as FP32 pairs
 //   [4 Jp, 4.5 Jp)  fixed-point shift S_j of column j (int)
-//   then 3 rows of Jp + 4 64-bit words: per-column fixed-point totals of a sweep's column
-//   partials and its row residual (word Jp); sweep s adds into row s mod 3.
+//   then 2 rows of Jp + 4 64-bit words: per-column fixed-point totals of the sweeps' column
+//   partials and their row residuals (word Jp); sweep s adds into row s mod 2.
 // The totals are sums of integers, the same in any order, so every CTA reads the same column
 // sums whatever the number of CTAs or the order in which partitions arrive.
+//
+// The words carry their own completion: each partition adds its value plus 1 << 56, and a
+// reader, which knows what the word held when the row was last complete, has the sweep's total
+// once the difference counts all V partitions (V <= 152, a sweep's values stay below 2^56).  So
+// no barrier stands between the sweep and the column update, and nothing is cleared.  A row is
+// added to again two sweeps later, by a CTA that has seen the other row complete, to which
+// every CTA has added after it read this one.
 static constexpr int FX_BITS = 40;   // a column total of q^_j is about 2^40 units
+static constexpr int FX_TOP = 48;    // partials (and totals) from 2^48 on go to the exact path
 static constexpr int FX_ERR = 50;    // row residuals in units of 2^-50
-__host__ __device__ constexpr size_t gstate_words(int Jp) { return (size_t)Jp * 15 / 2 + 12; }
+static constexpr int FX_COUNT = 56;  // bit position of the partition count
+__host__ __device__ constexpr size_t gstate_words(int Jp) { return (size_t)Jp * 13 / 2 + 8; }
 __host__ __device__ constexpr size_t gstate_bytes(int Jp) { return 8 * gstate_words(Jp); }
 __device__ __forceinline__ float2* gs_lq2(double* G, int Jp) { return reinterpret_cast<float2*>(G + 3 * (size_t)Jp); }
 __device__ __forceinline__ int* gs_sx(double* G, int Jp) { return reinterpret_cast<int*>(G + 4 * (size_t)Jp); }
@@ -423,9 +432,17 @@ struct SkShared {
     float errf[16];         // per-team row residuals
     double sh_sum[24][2];   // per-warp setup sums (up to 24 consumer warps)
     int s_dec, s_ok, s_bad;
+    int flags[2];                    // of a sweep, by parity: EXACT, BAD and LATE below
+    unsigned long long s_err;        // total of the row residuals
     volatile int s_stop;    // consumers -> producer: stop streaming
     uint32_t tmem;          // tensor-memory address of the column potentials (see G_to_tmem)
     int pend[VMAX + 1];     // stage blocks (from the CTA's first row) at which its partitions end
+};
+
+enum : int {
+    SK_EXACT = 1,  // some column's total has to be summed from the partials
+    SK_BAD = 2,    // and one of those lost its mass
+    SK_LATE = 4,   // a wait for the totals gave up
 };
 
 // The CTAs that solve one instance together: nb CTAs, this one is number b.  `bar` counts
@@ -1024,7 +1041,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             const int sx = FX_BITS - (int)floor(lq);
             SX[j] = sx <= 126 ? sx : 0;
         }
-        for (int t = (b * NCW + warp) * 32 + lane; t < 3 * (Jp + 4); t += nw * 32) ACC[t] = 0ull;
+        for (int t = (b * NCW + warp) * 32 + lane; t < 2 * (Jp + 4); t += nw * 32) ACC[t] = 0ull;
         const float inv_sp_f = (float)(1.0 / sp);
         for (int r = tid; r < nrow; r += NC) Ps[r] *= inv_sp_f;  // p^_i
         bar_named(CONS_BAR, NC);
@@ -1345,8 +1362,21 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
 
     // ---- sweeps 2, 3, ...: one read of C and one ex2 per cell -----------------------------
     // Each partition adds its column partials (and row residual) as fixed-point integers into
-    // the row of totals of this sweep; after the one grid barrier of the iteration every CTA
-    // reads the totals and forms all column updates itself in its shared-memory copy of G.
+    // the row of totals of this sweep; every CTA waits for the totals themselves and forms all
+    // column updates in its shared-memory copy of G.
+    //
+    // The sync bounds small instances (it is half of an iteration up to 20,000 x 400) and idles
+    // HBM in large ones.  A grid barrier cost three dependent trips through L2 (the adds have to
+    // land before the arrival is released, the arrival, the totals); waiting on the counted
+    // totals costs one: 1000 x 50 245 -> 206 us, 5,000 x 128 warm 169 -> 155, 12,347 x 1,021
+    // packed 444 -> 426, 50,000 x 800 982 -> 964.
+    constexpr int UC = (4 * TT * VPT + NC - 1) / NC;  // columns a thread looks after: tid + NC u
+    constexpr int CU = UC < 3 ? UC : 3;               // and how many at a time
+    static_assert(UC <= 32, "one mask word");
+    unsigned long long prev[2][UC], prev_err[2] = {0ull, 0ull};  // the rows' words when last complete
+#pragma unroll
+    for (int u = 0; u < UC; ++u) prev[0][u] = prev[1][u] = 0ull;
+    if (tid == 0) sh->flags[0] = sh->flags[1] = 0;  // a barrier follows (G_to_tmem)
     constexpr int RPP = rows_per_pass<TW, VPT, EUC>();
     // a team's rows of a block come in pairs when there is an even number of them; otherwise a
     // step takes two blocks, if the ring has stages to spare for that
@@ -1355,7 +1385,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
     const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
     for (int s = 2;; ++s) {
-        unsigned long long* acc_s = ACC + (size_t)(s % 3) * (Jp + 4);
+        unsigned long long* acc_s = ACC + (size_t)(s & 1) * (Jp + 4);
         const float2* Fold = Fs + ((s - 1) & 1) * S.rmax;  // F'^(s-1)
         float2* Fnew = Fs + (s & 1) * S.rmax;
         f32x2 acc[VPT][2];
@@ -1408,122 +1438,201 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             }
             kb += nblk;
           }
-            // end of partition vp: its column partials (teams in order) and row residual.  The
-            // FP32 partial is kept for the exact path and added to the column's total as
-            // round(partial 2^S_j); a partial too large for the total marks the column.
+            // end of partition vp: its column partials (teams in order, as cta_col_sum) and row
+            // residual.  The FP32 partial is kept for the exact path and added to the column's
+            // total as round(partial 2^S_j); one too large for the total adds 2^FX_TOP, which
+            // sends the column there.
             if (tm.tl == 0) errf[tm.team] = errt;
-            float* cp = P.colpart + (int64_t)vp * Jp;
-            float4 part[VPT];
+            int sx[CU];  // of this thread's first columns: on the way while the teams merge
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                const float2 a = unpack2(acc[v][0]), b = unpack2(acc[v][1]);
-                part[v] = make_float4(a.x, a.y, b.x, b.y);
+            for (int u = 0; u < CU; ++u) sx[u] = tid + u * NC < J ? __ldcg(SX + tid + u * NC) : 0;
+            if (tm.team < HALF) {
+#pragma unroll
+                for (int v = 0; v < VPT; ++v) {
+                    const int col = 4 * (tm.tl + TT * v);
+                    if (col < Jp) *reinterpret_cast<ulonglong2*>(comb + tm.team * Jp + col) = make_ulonglong2(acc[v][0], acc[v][1]);
+                }
             }
-            cta_col_sum<TW, VPT>(comb, part, J, Jp, tm, [&](int j, float sum) {
-                cp[j] = sum;
-                const int sx = SX[j];
-                const float x = ldexpf(sum, sx);
-                if (sx != 0 && x < 0x1p55f) atomicAdd(acc_s + j, (unsigned long long)__float2ull_rn(x));
-                else atomicOr(acc_s + j, 1ull << 63);
-            });
-            if (tid == 0) {
+            bar_named(CONS_BAR, NC);
+            if (tid == 0) {  // its team is done; the other half merges meanwhile
                 float2 e = make_float2(errf[0], 0.f);
                 for (int t = 1; t < NTEAMS; ++t) e = df_add(e, errf[t]);
-                atomicAdd(acc_s + Jp, (unsigned long long)__float2ull_rn(ldexpf(e.x + e.y, FX_ERR)));
-                s_bad = 0;
+                // at most 2^51 in all for a plan of unit mass; a broken plan's must not reach the count
+                const float x = ldexpf(e.x + e.y, FX_ERR);
+                atomicAdd(acc_s + Jp, (1ull << FX_COUNT) + (x < 0x1p52f ? __float2ull_rn(x) : 1ull << FX_TOP));
             }
+            if (tm.team >= HALF) {
+#pragma unroll
+                for (int v = 0; v < VPT; ++v) {
+                    const int col = 4 * (tm.tl + TT * v);
+                    if (col < Jp) {
+                        ulonglong2* d = reinterpret_cast<ulonglong2*>(comb + (tm.team - HALF) * Jp + col);
+                        const ulonglong2 o = *d;
+                        *d = make_ulonglong2(add2(o.x, acc[v][0]), add2(o.y, acc[v][1]));
+                    }
+                }
+            }
+            bar_named(CONS_BAR, NC);
+            float* cp = P.colpart + (int64_t)vp * Jp;
+            auto add_total = [&](int j, int sxj) {
+                float sum = comb[j];
+                for (int t = 1; t < HALF; ++t) sum += comb[t * Jp + j];
+                cp[j] = sum;
+                const float x = sum * __int_as_float((sxj + 127) << 23);  // S_j <= 126; 0 for "never"
+                const bool fits = sxj != 0 && x < (float)(1ull << FX_TOP);
+                atomicAdd(acc_s + j, (1ull << FX_COUNT) + (fits ? __float2ull_rn(x) : 1ull << FX_TOP));
+            };
+#pragma unroll
+            for (int u = 0; u < CU; ++u)
+                if (tid + u * NC < J) add_total(tid + u * NC, sx[u]);
+            for (int j = tid + CU * NC; j < J; j += NC) add_total(j, __ldcg(SX + j));
 #pragma unroll
             for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
             errt = 0.f;
-            if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // errf is read by thread 0 above
+            if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // comb and errf are free again
         }
         tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
-        // the constant per-column values of this thread's first round of column updates are
-        // loaded before the barrier, so only the totals cross L2 after it
-        constexpr int CU = 3;
-        float2 lq0[CU];
-        int sx0[CU];
-#pragma unroll
-        for (int u = 0; u < CU; ++u) {
-            const int j = tid + u * NC;
-            lq0[u] = j < J ? __ldcg(LQ2 + j) : make_float2(0.f, 0.f);
-            sx0[u] = j < J ? __ldcg(SX + j) : 0;
-        }
-        OTA_BARRIER();
-        // Loop test on pi^(s-1): every thread reads the same total of the row residuals.
-        const double ed = (double)__ldcg(acc_s + Jp) * 0x1p-50;
-        const bool conv = ed <= stop_tol(P.tol);
-        if (conv || s - 1 >= P.max_iter) {
-            if (b == 0 && tid == 0) {
-                P.st->iters = s - 1;
-                P.st->err = ed;
-                P.st->converged = conv;
-            }
-            if (P.F_out)
-                for (int r = tid; r < nrow; r += NC) P.F_out[r0 + r] = Fold[r];
-            *ret_par = (s - 1) & 1;
-            if (P.fpart) sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
-            if (tid == 0) s_stop = 1;
-            return true;
-        }
         // G^s_j = G^(s-1)_j + log2 q^_j - log2 s_j, every column in every CTA (FP32 pairs).  The
-        // sum s_j is the fixed-point total T_j 2^-S_j; a marked column, or one whose total is
-        // too small to carry 30 bits, is summed exactly from the partitions' FP32 partials.
-        {
-            double* Gnew = P.G + (s & 1) * Jp;
-            int bad = 0;
-            // CU columns a thread per round: all loads of a round first (one trip to L2), then
-            // the arithmetic
-            for (int j0 = tid; j0 < J; j0 += CU * NC) {
-                unsigned long long T[CU];
-                float2 lq[CU];
-                int sx[CU];
+        // sum s_j is the fixed-point total T_j 2^-S_j; a column whose total is too large or too
+        // small to carry 30 bits is summed exactly from the partitions' FP32 partials instead.
+        unsigned exact = 0;  // of this thread's columns
+        int* flags = &sh->flags[s & 1];
+        for (int u0 = 0; u0 < UC; u0 += CU) {
+            unsigned long long T[CU], was[CU];
+            float2 lq[CU];
+            int sx[CU];
+#pragma unroll
+            for (int u = 0; u < CU; ++u) {  // constants of the columns, on the way during the wait
+                const int j = tid + (u0 + u) * NC;
+                const bool in = u0 + u < UC && j < J;
+                lq[u] = in ? __ldcg(LQ2 + j) : make_float2(0.f, 0.f);
+                sx[u] = in ? __ldcg(SX + j) : 0;
+                was[u] = in ? prev[s & 1][u0 + u] : 0ull;
+                T[u] = 0ull;
+            }
+            const bool first = u0 == 0;
+            long long n = 0;
+            for (;;) {  // until every partition's addition to this thread's words has arrived
+                bool all = true;
+                unsigned long long A[CU], Ae = 0ull;
 #pragma unroll
                 for (int u = 0; u < CU; ++u) {
-                    const int j = j0 + u * NC;
-                    T[u] = j < J ? __ldcg(acc_s + j) : 0ull;
-                    lq[u] = j0 == tid ? lq0[u] : (j < J ? __ldcg(LQ2 + j) : make_float2(0.f, 0.f));
-                    sx[u] = j0 == tid ? sx0[u] : (j < J ? __ldcg(SX + j) : 0);
+                    const int j = tid + (u0 + u) * NC;
+                    A[u] = u0 + u < UC && j < J ? ld_relaxed_u64(acc_s + j) : was[u] + ((unsigned long long)V << FX_COUNT);
                 }
+                if (first && tid == 0) Ae = ld_relaxed_u64(acc_s + Jp);
 #pragma unroll
                 for (int u = 0; u < CU; ++u) {
-                    const int j = j0 + u * NC;
-                    if (j >= J) break;
-                    float2 ls;
-                    if (!(T[u] >> 63) && T[u] >= (1ull << 30)) {
-                        const float th = __ull2float_rn(T[u]);
-                        const float tl = (float)((long long)T[u] - (long long)__float2ull_rn(th));
-                        ls = df_log2(make_float2(th, tl));
-                        ls.x -= (float)sx[u];
-                    } else {
-                        float2 sum = make_float2(0.f, 0.f);
-                        for (int v = 0; v < V; ++v) sum = df_add(sum, __ldcg(P.colpart + (int64_t)v * Jp + j));
-                        if (!(sum.x > 0.f) || !isfinite(sum.x)) {
-                            bad = 1;
-                            continue;
-                        }
-                        ls = df_log2(sum);
+                    T[u] = A[u] - was[u];
+                    all = all && (T[u] >> FX_COUNT) == (unsigned long long)V;
+                }
+                if (first && tid == 0) {
+                    const unsigned long long D = Ae - prev_err[s & 1];
+                    all = all && (D >> FX_COUNT) == (unsigned long long)V;
+                    if (all) {
+                        prev_err[s & 1] = Ae;
+                        sh->s_err = D & ((1ull << FX_COUNT) - 1);
                     }
-                    const float2 d = df_add2(lq[u], make_float2(-ls.x, -ls.y));
-                    const float2 Gn = df_add2(make_float2(Gs[j], Gs[Jp + j]), d);
+                }
+                if (all) {
+#pragma unroll
+                    for (int u = 0; u < CU; ++u)
+                        if (u0 + u < UC) prev[s & 1][u0 + u] = A[u];
+                    break;
+                }
+                ++n;
+                if ((n & 63) == 0 && ld_volatile_i32(g.abort) != DEV_OK) {
+                    atomicOr(flags, SK_LATE);
+                    break;
+                }
+                if (n > P.spin) {
+                    atomicCAS(g.abort, DEV_OK, DEV_ETIMEOUT);
+                    atomicOr(flags, SK_LATE);
+                    break;
+                }
+                if (n > 256) __nanosleep(32);
+            }
+            if (first) {
+                bar_named(CONS_BAR, NC);
+                if (*(volatile int*)flags & SK_LATE) {
+                    if (tid == 0) s_stop = 1;
+                    return false;
+                }
+                if (tid == 0) sh->flags[(s + 1) & 1] = 0;  // read last before the barrier that ended sweep s - 1
+                // Loop test on pi^(s-1): every CTA reads the same total of the row residuals.
+                const double ed = (double)sh->s_err * 0x1p-50;
+                const bool conv = ed <= stop_tol(P.tol);
+                if (conv || s - 1 >= P.max_iter) {
+                    if (b == 0 && tid == 0) {
+                        P.st->iters = s - 1;
+                        P.st->err = ed;
+                        P.st->converged = conv;
+                    }
+                    if (s > 2)  // the FP64 copy of G^(s-1) (G^1 is there already), each column once
+                        for (int j = b * NC + tid; j < J; j += nb * NC)
+                            P.G[((s - 1) & 1) * Jp + j] = (double)Gs[j] + (double)Gs[Jp + j];
+                    if (P.F_out)
+                        for (int r = tid; r < nrow; r += NC) P.F_out[r0 + r] = Fold[r];
+                    *ret_par = (s - 1) & 1;
+                    if (P.fpart) sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
+                    if (tid == 0) s_stop = 1;
+                    return true;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < CU; ++u) {
+                const int j = tid + (u0 + u) * NC;
+                T[u] &= (1ull << FX_COUNT) - 1;
+                const bool in = u0 + u < UC && j < J;
+                const bool ok = T[u] >= (1ull << 30) && T[u] < (1ull << FX_TOP);
+                const float th = __ull2float_rn(T[u]);
+                const float tl = (float)((long long)T[u] - (long long)__float2ull_rn(th));
+                float2 ls = df_log2(make_float2(ok ? th : 1.f, ok ? tl : 0.f));
+                ls.x -= (float)sx[u];
+                const float2 d = df_add2(lq[u], make_float2(-ls.x, -ls.y));
+                const int jr = in ? j : 0;
+                const float2 Gn = df_add2(make_float2(Gs[jr], Gs[Jp + jr]), d);
+                if (in && ok) {
                     Gs[j] = Gn.x;
                     Gs[Jp + j] = Gn.y;
-                    if ((j >> 5) % nb == b) Gnew[j] = (double)Gn.x + (double)Gn.y;  // the FP64 copy, once
                 }
+                if (in && !ok) exact |= 1u << (u0 + u);
             }
-            // this CTA's share of clearing the totals of sweep s + 2 (last read before this
-            // iteration's barrier; next written after the next one)
-            unsigned long long* acc_z = ACC + (size_t)((s + 2) % 3) * (Jp + 4);
-            for (int t = b * NC + tid; t < Jp + 4; t += nb * NC) acc_z[t] = 0ull;
-            if (bad) atomicOr(&s_bad, 1);
-            bar_named(CONS_BAR, NC);
-            if (s_bad) {  // every CTA sees the same totals and takes the same decision
+        }
+        if (exact) atomicOr(flags, SK_EXACT);
+        bar_named(CONS_BAR, NC);
+        const int fl = *(volatile int*)flags;
+        if (fl & SK_LATE) {
+            if (tid == 0) s_stop = 1;
+            return false;
+        }
+        if (fl) {  // every CTA sees the same totals and comes here or not; the partials need a barrier
+            OTA_BARRIER();
+            int bad = 0;
+            for (int u = 0; u < UC; ++u) {
+                if (!(exact >> u & 1u)) continue;
+                const int j = tid + u * NC;
+                float2 sum = make_float2(0.f, 0.f);
+                for (int v = 0; v < V; ++v) sum = df_add(sum, __ldcg(P.colpart + (int64_t)v * Jp + j));
+                if (!(sum.x > 0.f) || !isfinite(sum.x)) {
+                    bad = 1;
+                    continue;
+                }
+                const float2 ls = df_log2(sum);
+                const float2 d = df_add2(__ldcg(LQ2 + j), make_float2(-ls.x, -ls.y));
+                const float2 Gn = df_add2(make_float2(Gs[j], Gs[Jp + j]), d);
+                Gs[j] = Gn.x;
+                Gs[Jp + j] = Gn.y;
+            }
+            if (bad) atomicOr(flags, SK_BAD);
+            OTA_BARRIER();  // the partials are read before any CTA writes the next sweep's
+            if (*(volatile int*)flags & SK_BAD) {  // the same decision in every CTA
                 if (tid == 0) atomicCAS(status, DEV_OK, DEV_ENUMERIC);
                 if (tid == 0) s_stop = 1;
                 return false;
             }
-            G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
         }
+        G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
     }
 #undef OTA_BARRIER_CHECK
 #undef OTA_BARRIER

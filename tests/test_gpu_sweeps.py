@@ -69,3 +69,50 @@ def test_fp64_tile_edges(ctx, shape):
     cost, rho, _, _ = oracle.finalize(C, f, g, p, q, 0.05)
     assert res.transport_cost == pytest.approx(cost, rel=1e-12)
     np.testing.assert_allclose(res.rrh_load.cpu().numpy(), rho, rtol=1e-12)
+
+
+def _crowded(kind, I, J):
+    """A column whose sum leaves the range of the fixed-point totals: a target of 1e-30, or a
+    target of 1e-6 for the column that nearly all the mass first goes to."""
+    rng = np.random.Generator(np.random.PCG64(I + J))
+    C = rng.uniform(0.0, 1.0, (I, J)).astype(np.float32)
+    p = rng.lognormal(0.0, 1.0, I)
+    q = rng.uniform(0.5, 1.5, J)
+    q[J // 2] = 1e-30 if kind == "tiny" else 1e-6
+    if kind == "crowded":
+        C[:, J // 2] -= 2.0
+    return C, (p / p.sum()).astype(np.float32), (q / q.sum()).astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["tiny", "crowded"])
+@pytest.mark.parametrize("shape", [(300, 50), (900, 1300)])
+@pytest.mark.parametrize("iters", [2, 3, 6])
+def test_column_totals_out_of_range(ctx, kind, shape, iters):
+    """Such columns are summed from the partitions' partials; iterates equal the oracle's."""
+    I, J = shape
+    C, p, q = _crowded(kind, I, J)
+    res = ctx.solve_cost(torch.from_numpy(C).cuda(), torch.from_numpy(p).cuda(), torch.from_numpy(q).cuda(), 0.1, tol=0.0,
+                         max_iter=iters, want_pi=True)
+    C64 = C.astype(np.float64)
+    f, g, _, _ = oracle.sinkhorn(C64, p, q, 0.1, 0.0, iters)
+    pi = oracle.plan(C64, f, g, 0.1)
+    err = np.abs(res.pi.cpu().numpy().astype(np.float64) - pi)
+    assert (err <= 2e-5 * pi + 1e-12).all()
+
+
+@pytest.mark.parametrize("kind", ["tiny", "crowded"])
+def test_group_with_idle_ctas(kind):
+    """A group of CTAs larger than the instance's row partitions: the idle ones follow the same
+    totals (and the same detours to the partials) and the result is the single solver's."""
+    from paper_1805_01559_gb300 import binding
+    I, J = 200, 52
+    C, p, q = _crowded(kind, I, J)
+    t = [torch.from_numpy(x).cuda() for x in (C, p, q)]
+    with binding.Context(0) as c:
+        one = c.solve_cost(*t, 0.1, tol=0.0, max_iter=6)
+        n = torch.cuda.get_device_properties(0).multi_processor_count
+        c.set_tuning(binding.bucket(I, J), n, 24576)
+        inst = [binding.Instance(C=t[0], p=t[1], q=t[2], eps=0.1, tol=0.0, max_iter=6) for _ in range(3)]
+        c.solve_batched(inst)
+        for x in inst:
+            assert torch.equal(x.f, one.f) and torch.equal(x.g, one.g)
