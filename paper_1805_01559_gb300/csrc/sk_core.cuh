@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "ot_common.cuh"
 
 namespace ota {
@@ -434,6 +436,7 @@ struct SkShared {
     int s_dec, s_ok, s_bad;
     int flags[2];                    // of a sweep, by parity: EXACT, BAD and LATE below
     unsigned long long s_err;        // total of the row residuals
+    unsigned long long werr[16];     // per team, of the current partition
     volatile int s_stop;    // consumers -> producer: stop streaming
     uint32_t tmem;          // tensor-memory address of the column potentials (see G_to_tmem)
     int pend[VMAX + 1];     // stage blocks (from the CTA's first row) at which its partitions end
@@ -702,7 +705,7 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
 }
 
 // Sums of R rows' per-lane values over the team, each in the order of team_reduce; every lane
-// gets all R.  Two rows share one butterfly: after the first exchange the lower half-warp
+// gets all R.  The rows share one butterfly: after the first exchange the lower half-warp
 // holds row 0's sums and the upper half row 1's (the same pairs are added), so two rows take
 // the shuffles of one plus one exchange, and wider teams one named barrier.
 template <int TW, int R>
@@ -802,8 +805,8 @@ __host__ __device__ constexpr int rows_per_pass() {
 }
 
 // One plan-scale pass of a team over R rows of C at once (row[k]: the staged row, or unused
-// when EUC with the device at dxy[k]): t_ij = 2^(F'_i + G_j - k C_ij), the row sums r_i, the
-// row update and residual, and the column accumulators acc += t p^ / r, row 0 before row 1.
+// when EUC with the device at dxy[k]): t_ij = 2^(F'_i + G_j - k C_ij), the row sums r_i (left
+// in Fnew for row_updates) and the column accumulators acc += t p^ / r, row 0 before row 1.
 // Bound by instruction issue and by the latency of a row's chain (shared-memory loads, ex2,
 // the team sum, the update) once C streams: two rows in flight hide one chain behind the
 // other and share the loads of G, and packed arithmetic halves the instructions of the
@@ -811,20 +814,19 @@ __host__ __device__ constexpr int rows_per_pass() {
 // with the chunk count of a lane fitted to the row for wide teams too).  Every operation
 // rounds as for one row at a time, so results are the same bit for bit.
 template <int TW, int VPT, bool EUC, int R>
-__device__ __forceinline__ void sweep_rows(const float* const (&row)[R], const float2 (&dxy)[R], uint32_t tG, int J,
+__device__ __forceinline__ void sweep_rows(const float* (&row)[R], const float2 (&dxy)[R], uint32_t tG, int J,
                                            int Jp, const float* rxs, f32x2 nk_hi, f32x2 nk_lo, const float2* Fold,
                                            float2* Fnew, const float* Ps, const int (&lr)[R], float* red, int nteams,
-                                           const Team<TW>& tm, int& par, f32x2 (&acc)[VPT][2], float& errt) {
+                                           const Team<TW>& tm, int& par, f32x2 (&acc)[VPT][2]) {
     constexpr int TT = 32 * TW;
     __syncwarp();
     f32x2 t[R][VPT][2], Fh[R], Fl[R];
-    float2 F[R];
     float rsum[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) {
-        F[k] = Fold[lr[k]];
-        Fh[k] = pack2(F[k].x, F[k].x);
-        Fl[k] = pack2(F[k].y, F[k].y);
+        const float2 F = Fold[lr[k]];
+        Fh[k] = pack2(F.x, F.x);
+        Fl[k] = pack2(F.y, F.y);
         rsum[k] = 0.f;
     }
 #pragma unroll
@@ -834,9 +836,14 @@ __device__ __forceinline__ void sweep_rows(const float* const (&row)[R], const f
         const bool all_in = chunk_inside<TW, VPT>(v);
         const int at = 4 * (tm.tl + TT * v);
         const int col = all_in || at < J ? at : 0;
-        float4 g4, l4;
-        tmem_ld8(tG + 8 * v, g4, l4);
-        const f32x2 gh[2] = {pack2(g4.x, g4.y), pack2(g4.z, g4.w)}, gl[2] = {pack2(l4.x, l4.y), pack2(l4.z, l4.w)};
+        uint32_t w[8];
+        tmem_ld8(tG + 8 * v, w);
+        f32x2 gh[2], gl[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            gh[h] = pack2(__uint_as_float(w[2 * h]), __uint_as_float(w[2 * h + 1]));
+            gl[h] = pack2(__uint_as_float(w[4 + 2 * h]), __uint_as_float(w[5 + 2 * h]));
+        }
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             f32x2 c[2];
@@ -866,32 +873,42 @@ __device__ __forceinline__ void sweep_rows(const float* const (&row)[R], const f
         }
     }
     team_sum_rows<TW, R>(rsum, red, nteams, tm, par);
-    float d[R];
 #pragma unroll
     for (int k = 0; k < R; ++k) {
-        const float ph = Ps[lr[k]];
-        errt = fmaf(ph, fabsf(rsum[k] - 1.0f), errt);
-        d[k] = __fdividef(ph, rsum[k]);
-    }
-    if constexpr (R == 1) {
-        // every lane forms the update (no divergent branch); one lane stores it
-        const float2 Fn = df_sub(F[0], log2_corr(rsum[0]));
-        if (tm.tl == 0) Fnew[lr[0]] = Fn;
-    } else {  // the lower half-warp forms row 0's update, the upper row 1's
-        const bool up = tm.lane >= 16;
-        const float2 Fu = up ? F[1] : F[0];
-        const float2 Fn = df_sub(Fu, log2_corr(up ? rsum[1] : rsum[0]));
-        if ((tm.lane & 15) == 0 && tm.wit == 0) Fnew[up ? lr[1] : lr[0]] = Fn;
-    }
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-        const f32x2 dk = pack2(d[k], d[k]);
+        if (tm.tl == 0) Fnew[lr[k]].x = rsum[k];
+        const float d = __fdividef(Ps[lr[k]], rsum[k]);
+        const f32x2 dk = pack2(d, d);
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             acc[v][0] = fma2(t[k][v][0], dk, acc[v][0]);
             acc[v][1] = fma2(t[k][v][1], dk, acc[v][1]);
         }
     }
+}
+
+// The row updates F'^s = F'^(s-1) - log2 r of a team's rows lr0, lr0 + step, ... below `end`
+// (their sums in Fnew), a lane a row, and the team's part of the residual sum p^ |r - 1| in
+// units of 2^-FX_ERR, an integer so that its order does not matter.  Called by the warp that
+// stored the sums.  Done for every row by a whole warp inside the sweep, this took 270 of the
+// 1,370 cycles of a row of 800 columns, and FP64 in the loop test 1,000 cycles of every sync;
+// without both 1000 x 50 went from 207 to 190 us, 5,000 x 128 warm from 155 to 144, 48 ragged
+// instances from 13.1 to 12.7 ms.
+__device__ __forceinline__ unsigned long long row_updates(const float2* Fold, float2* Fnew, const float* Ps, int lr0,
+                                                          int step, int end, int lane) {
+    unsigned long long e = 0ull;
+    __syncwarp();
+    for (int lr = lr0 + step * lane; lr < end; lr += step * 32) {
+        const float r = Fnew[lr].x;
+        Fnew[lr] = df_sub(Fold[lr], log2_corr(r));
+        const float x = Ps[lr] * fabsf(r - 1.0f) * 0x1p50f;
+        e += x < 0x1p52f ? __float2ull_rn(x) : 1ull << 52;
+    }
+    const unsigned m = (1u << 18) - 1;
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)e & m);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(e >> 18) & m);
+    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(e >> 36));
+    e = a + ((unsigned long long)b << 18) + ((unsigned long long)c << 36);
+    return e < (1ull << 52) ? e : 1ull << 52;
 }
 
 // The consumer warps' part of one solve (Algorithm 1 on the CTA's partitions, rows [r0, r1)):
@@ -916,7 +933,6 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     float* ring = reinterpret_cast<float*>(dyn + S.off_ring);  // [stages][stage_floats]
     const float* rxs = ring;  // Euclidean cost: RRH x then y coordinates [2][Jp]
     float* red = sh->red;
-    float* errf = sh->errf;
     double(*sh_sum)[2] = sh->sh_sum;
     int& s_bad = sh->s_bad;
     volatile int& s_stop = sh->s_stop;
@@ -1377,10 +1393,13 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
 #pragma unroll
     for (int u = 0; u < UC; ++u) prev[0][u] = prev[1][u] = 0ull;
     if (tid == 0) sh->flags[0] = sh->flags[1] = 0;  // a barrier follows (G_to_tmem)
+    // the loop test's bound in the residual's units (totals stay below 2^FX_COUNT)
+    const double stop_d = stop_tol(P.tol) * 0x1p50;
+    const unsigned long long stop_units = stop_d < 0x1p56 ? (unsigned long long)stop_d : 1ull << FX_COUNT;
     constexpr int RPP = rows_per_pass<TW, VPT, EUC>();
-    // a team's rows of a block come in pairs when there is an even number of them; otherwise a
-    // step takes two blocks, if the ring has stages to spare for that
-    const int step_blocks = RPP == 2 && (S.rpt & 1) && S.stages >= 4 ? 2 : 1;
+    // a step takes two blocks where a team's rows of one do not fill its passes, if the ring has
+    // stages to spare for that
+    const int step_blocks = S.rpt % RPP != 0 && S.stages >= 4 ? 2 : 1;
     const uint32_t tG = tmem_G<TW, VPT>(sh->tmem, tm);
     G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
     const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
@@ -1391,10 +1410,10 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         f32x2 acc[VPT][2];
 #pragma unroll
         for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
-        float errt = 0.f;  // every lane of a team holds the same value
         int kb = 0;
         for (int vp = v0; vp < v1; ++vp) {
           const int vend = pend[vp];
+          const int kb0 = kb;
           while (kb < vend) {
             // a step: one stage block, or two when a team's rows in a block do not pair up
             const int nblk = min(step_blocks, vend - kb);
@@ -1414,22 +1433,29 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             auto staged = [&](int q) {
                 return q < S.rpt ? stage0 + (size_t)(NTEAMS * q) * P.ld : stage1 + (size_t)(NTEAMS * (q - S.rpt)) * P.ld;
             };
-            for (int q = 0; q < nq; q += RPP) {
-                if constexpr (RPP == 2) {
+            auto pass = [&](auto rows, int q) {
+                constexpr int R = decltype(rows)::value;
+                int lr[R];
+                const float* row[R];
+                float2 dxy[R];
+#pragma unroll
+                for (int k = 0; k < R; ++k) {
+                    lr[k] = lr0 + NTEAMS * (q + k);
+                    row[k] = staged(q + k);
+                    dxy[k] = EUC ? __ldg(P.dev_xy + r0 + lr[k]) : make_float2(0.f, 0.f);
+                }
+                sweep_rows<TW, VPT, EUC, R>(row, dxy, tG, J, Jp, rxs, nk_hi, nk_lo, Fold, Fnew, Ps, lr, red, NTEAMS, tm, par,
+                                            acc);
+            };
+            for (int q = 0; q < nq;) {
+                if constexpr (RPP == 2)
                     if (q + 1 < nq) {
-                        const int lr[2] = {lr0 + NTEAMS * q, lr0 + NTEAMS * (q + 1)};
-                        const float* const row[2] = {staged(q), staged(q + 1)};
-                        const float2 dxy[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                        sweep_rows<TW, VPT, EUC, 2>(row, dxy, tG, J, Jp, rxs, nk_hi, nk_lo, Fold, Fnew, Ps, lr, red, NTEAMS,
-                                                    tm, par, acc, errt);
+                        pass(std::integral_constant<int, 2>(), q);
+                        q += 2;
                         continue;
                     }
-                }
-                const int lr[1] = {lr0 + NTEAMS * q};
-                const float* const row[1] = {staged(q)};
-                const float2 dxy[1] = {EUC ? __ldg(P.dev_xy + r0 + lr[0]) : make_float2(0.f, 0.f)};
-                sweep_rows<TW, VPT, EUC, 1>(row, dxy, tG, J, Jp, rxs, nk_hi, nk_lo, Fold, Fnew, Ps, lr, red, NTEAMS, tm,
-                                            par, acc, errt);
+                pass(std::integral_constant<int, 1>(), q);
+                ++q;
             }
             __syncwarp();
             if (!EUC && lane == 0) {
@@ -1442,7 +1468,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             // residual.  The FP32 partial is kept for the exact path and added to the column's
             // total as round(partial 2^S_j); one too large for the total adds 2^FX_TOP, which
             // sends the column there.
-            if (tm.tl == 0) errf[tm.team] = errt;
+            if (tm.wit == 0) {
+                const unsigned long long e =
+                    row_updates(Fold, Fnew, Ps, kb0 * rs_ + tm.team, NTEAMS, min(vend * rs_, nrow), lane);
+                if (lane == 0) sh->werr[tm.team] = e;
+            }
             int sx[CU];  // of this thread's first columns: on the way while the teams merge
 #pragma unroll
             for (int u = 0; u < CU; ++u) sx[u] = tid + u * NC < J ? __ldcg(SX + tid + u * NC) : 0;
@@ -1455,11 +1485,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             }
             bar_named(CONS_BAR, NC);
             if (tid == 0) {  // its team is done; the other half merges meanwhile
-                float2 e = make_float2(errf[0], 0.f);
-                for (int t = 1; t < NTEAMS; ++t) e = df_add(e, errf[t]);
+                unsigned long long e = 0ull;
+#pragma unroll
+                for (int t = 0; t < NTEAMS; ++t) e += sh->werr[t];
                 // at most 2^51 in all for a plan of unit mass; a broken plan's must not reach the count
-                const float x = ldexpf(e.x + e.y, FX_ERR);
-                atomicAdd(acc_s + Jp, (1ull << FX_COUNT) + (x < 0x1p52f ? __float2ull_rn(x) : 1ull << FX_TOP));
+                atomicAdd(acc_s + Jp, (1ull << FX_COUNT) + (e < (1ull << 52) ? e : 1ull << FX_TOP));
             }
             if (tm.team >= HALF) {
 #pragma unroll
@@ -1488,8 +1518,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             for (int j = tid + CU * NC; j < J; j += NC) add_total(j, __ldcg(SX + j));
 #pragma unroll
             for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
-            errt = 0.f;
-            if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // comb and errf are free again
+            if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // comb and werr are free again
         }
         tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
         // G^s_j = G^(s-1)_j + log2 q^_j - log2 s_j, every column in every CTA (FP32 pairs).  The
@@ -1560,12 +1589,12 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 }
                 if (tid == 0) sh->flags[(s + 1) & 1] = 0;  // read last before the barrier that ended sweep s - 1
                 // Loop test on pi^(s-1): every CTA reads the same total of the row residuals.
-                const double ed = (double)sh->s_err * 0x1p-50;
-                const bool conv = ed <= stop_tol(P.tol);
+                // (in integers: FP64 in every warp would take a thousand cycles of every sync)
+                const bool conv = sh->s_err <= stop_units;
                 if (conv || s - 1 >= P.max_iter) {
                     if (b == 0 && tid == 0) {
                         P.st->iters = s - 1;
-                        P.st->err = ed;
+                        P.st->err = (double)sh->s_err * 0x1p-50;
                         P.st->converged = conv;
                     }
                     if (s > 2)  // the FP64 copy of G^(s-1) (G^1 is there already), each column once
