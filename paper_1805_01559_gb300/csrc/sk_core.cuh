@@ -230,6 +230,15 @@ __device__ __forceinline__ void euclid_row(float2 d, const float* rx, const floa
     }
 }
 
+// The sweeps read a CTA's rows round after round, so a matrix larger than L2 (129 MB) would
+// leave nothing of itself there for the next sweep.  The first L2_KEEP bytes of a CTA's rows
+// (80 MB over 152 SMs, 5/8 of L2) keep the normal eviction priority and the rest is marked to
+// be evicted first, so the kept part survives and is read from L2.  50,000 x 800 (160 MB):
+// 954 -> 880 us a solve, 48 ragged instances 12.7 -> 12.4 ms.  Kept parts from 60 to 100 MB and
+// the persisting priority (evict_last) instead of the normal one differ by 3% at most; the
+// persisting one would hold L2 against whatever runs next.
+static constexpr int64_t L2_KEEP = 80000000 / 152;
+
 // Producer: stream the CTA's row blocks sweep after sweep until the consumers raise s_stop,
 // then wait for every copy still in flight before leaving.
 template <typename T>
@@ -239,6 +248,8 @@ __device__ __forceinline__ void stream_rows_producer(const T* C, int64_t ld, int
                                                      long long spin) {
     const int nblk = (int)((r1 - r0 + S.rows_per_stage - 1) / S.rows_per_stage);
     uint32_t seq = 0;
+    const uint64_t keep = l2_policy_normal(), pass = l2_policy_first();
+    const int64_t keep_rows = L2_KEEP / (ld * (int64_t)sizeof(T));
     bool stop = (nblk <= 0);
     while (!stop) {
         for (int k = 0; k < nblk && !stop; ++k) {
@@ -262,7 +273,8 @@ __device__ __forceinline__ void stream_rows_producer(const T* C, int64_t ld, int
             const int rows = (int)min((int64_t)S.rows_per_stage, r1 - row0);
             const uint32_t bytes = (uint32_t)(rows * ld * (int64_t)sizeof(T));
             mbar_arrive_expect_tx(&full[st], bytes);
-            bulk_g2s(ring + (size_t)st * S.stage_floats, C + row0 * ld, bytes, &full[st]);
+            bulk_g2s(ring + (size_t)st * S.stage_floats, C + row0 * ld, bytes, &full[st],
+                     row0 - r0 < keep_rows ? keep : pass);
             ++seq;
         }
     }
