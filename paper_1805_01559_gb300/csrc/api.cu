@@ -115,6 +115,12 @@ void timing_collect(ot_assoc_ctx* ctx, int sweeps) {
     ctx->last_timings = t;
 }
 
+// What a cost set-up leaves on the device for the host: count of invalid rates, median.
+struct CostState {
+    unsigned long long bad;
+    double med[2];
+};
+
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Make a 16-byte-aligned copy of a strided FP32 matrix when it is not aligned already.
@@ -282,10 +288,10 @@ ot_status ot_assoc_build_cost_from_gains(ot_assoc_ctx* ctx, const float* G, int6
     cudaStream_t s = (cudaStream_t)stream;
     ot_status st = aligned_view(ctx, G, ld_g, I, (int)J, s, &G, &ld_g, SLOT_ALIGN);
     if (st) return st;
-    char* state = (char*)scratch(ctx, SLOT_MISC, 256, &st);
+    CostState* state = (CostState*)scratch(ctx, SLOT_MISC, sizeof(CostState), &st);
     if (st) return st;
-    unsigned long long* bad = (unsigned long long*)state;
-    double* med = (double*)(state + 64);
+    unsigned long long* bad = &state->bad;
+    double* med = state->med;
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "memset");
     st = launch_rates(ctx, G, ld_g, P, I, (int)J, N0, W_hz, R_out, ld_r, s, mu, C_out, ld_c, bad);
@@ -293,17 +299,14 @@ ot_status ot_assoc_build_cost_from_gains(ot_assoc_ctx* ctx, const float* G, int6
     if (!eps_out) return OT_OK;
     st = launch_median(ctx, C_out, I, J, ld_c, med, s);
     if (st) return st;
-    struct {
-        unsigned long long bad;
-        double med;
-    }* h = (decltype(h))host_staging(ctx, 64, &st);
+    CostState* h = (CostState*)host_staging(ctx, sizeof(CostState), &st);
     if (st) return st;
-    e = cudaMemcpyAsync(&h->bad, bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h->med, med, sizeof(double), cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(h, state, sizeof(CostState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "build_cost_from_gains");
     if (h->bad) return set_error(ctx, OT_EINVAL, "%llu rate entries are not finite and > 0", h->bad);
-    *eps_out = eps_rel * h->med;
+    if (h->med[1] != 0.0) return set_error(ctx, OT_ETIMEOUT, "median: a device-side wait exceeded its spin limit");
+    *eps_out = eps_rel * h->med[0];
     return OT_OK;
 }
 
@@ -338,10 +341,10 @@ ot_status ot_assoc_build_cost(ot_assoc_ctx* ctx, const float* R, int64_t ld_r, i
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     ot_status st = OT_OK;
-    char* state = (char*)scratch(ctx, SLOT_MISC, 256, &st);
+    CostState* state = (CostState*)scratch(ctx, SLOT_MISC, sizeof(CostState), &st);
     if (st) return st;
-    unsigned long long* bad = (unsigned long long*)state;
-    double* med = (double*)(state + 64);
+    unsigned long long* bad = &state->bad;
+    double* med = state->med;
     cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "memset");
     st = launch_cost(ctx, R, ld_r, I, (int)J, mu, C_out, ld_c, false, bad, s);
@@ -349,17 +352,14 @@ ot_status ot_assoc_build_cost(ot_assoc_ctx* ctx, const float* R, int64_t ld_r, i
     if (!eps_out) return OT_OK;
     st = launch_median(ctx, C_out, I, J, ld_c, med, s);
     if (st) return st;
-    struct {
-        unsigned long long bad;
-        double med;
-    }* h = (decltype(h))host_staging(ctx, 64, &st);
+    CostState* h = (CostState*)host_staging(ctx, sizeof(CostState), &st);
     if (st) return st;
-    e = cudaMemcpyAsync(&h->bad, bad, sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h->med, med, sizeof(double), cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(h, state, sizeof(CostState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "build_cost");
     if (h->bad) return set_error(ctx, OT_EINVAL, "%llu rate entries are not finite and > 0", h->bad);
-    *eps_out = eps_rel * h->med;
+    if (h->med[1] != 0.0) return set_error(ctx, OT_ETIMEOUT, "median: a device-side wait exceeded its spin limit");
+    *eps_out = eps_rel * h->med[0];
     return OT_OK;
 }
 
@@ -369,16 +369,16 @@ ot_status ot_assoc_median_f32(ot_assoc_ctx* ctx, const float* x, int64_t n, doub
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     ot_status st = OT_OK;
-    char* state = (char*)scratch(ctx, SLOT_MISC, 256, &st);
+    double* med = (double*)scratch(ctx, SLOT_MISC, 256, &st);
     if (st) return st;
-    double* med = (double*)(state + 64);
     st = launch_median(ctx, x, 1, n, n, med, s);
     if (st) return st;
     double* h = (double*)host_staging(ctx, 64, &st);
     if (st) return st;
-    cudaError_t e = cudaMemcpyAsync(h, med, sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(h, med, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "median");
+    if (h[1] != 0.0) return set_error(ctx, OT_ETIMEOUT, "median: a device-side wait exceeded its spin limit");
     *median_out = *h;
     return OT_OK;
 }

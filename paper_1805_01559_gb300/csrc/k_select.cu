@@ -2,19 +2,25 @@
 // eps = eps_rel * median(C) is how the benchmark configurations fix the regularization
 // strength of Eq. (5); the median of an even count is the mean of the two middle values.
 //
-// Method (all on the device, no host round trip):
-//   1. take s = 65536 entries at a fixed stride and select, exactly, the sample ranks
-//      s/2 -+ 6 sd (sd = sqrt(s)/2, the rank spread of a sample median): a bracket [lo, hi];
+// Method, in one cooperative launch:
+//   1. (from 2^20 entries on) every CTA takes the same 8192 entries, one at a hashed place of
+//      each 1/8192 of the data, and selects, exactly, the sample ranks s/2 -+ 4.5 sd
+//      (sd = sqrt(s)/2, the rank spread of a sample median): a bracket [lo, hi];
 //   2. one pass over all n entries counts those below lo and compacts those in [lo, hi]
-//      into a candidate buffer (a few percent of n);
+//      into a candidate buffer (about 5% of n);
 //   3. if both middle ranks fall inside the bracket and the candidates fit, select them
 //      among the candidates; otherwise select over all n entries.
-// Selection is a radix select (8 bits per pass) on order-preserving keys that tracks both
+// Selection is a radix select (11 bits per pass) on order-preserving keys that tracks both
 // middle ranks at once; among the candidates it starts below the leading bits that lo and
-// hi share, which spreads the first pass over many bins.  Each histogram pass ends with
-// its last block to finish (a counter, no waiting) picking the digits for the next pass.
-// The result is exact either way and does not depend on the order in which candidates were
-// compacted or blocks finished.
+// hi share.  Every CTA picks the digits itself from the grid's histogram, so a pass takes one
+// grid barrier.  The result is exact either way and does not depend on the order in which
+// candidates were compacted.
+//
+// What bounds it: the one pass over the data (160 MB on 50,000 x 800, 24 us of HBM), and below
+// about a million entries the trips between passes.  As eleven launches (four for the sample,
+// four for the candidates, at 7 to 10 us each) the median took 150 us of the 330 us that rates,
+// cost and median of 50,000 x 800 take, and half of the 100 us of a 1000 x 50 cell.
+// Now one launch of 79 us there (18 us on 1000 x 50): 323 -> 277 us and 99 -> 67 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -26,10 +32,12 @@
 
 namespace ota {
 
-static constexpr int RS_BITS = 8;
+static constexpr int RS_NT = 1024;               // threads of a CTA (one CTA an SM)
+static constexpr int RS_BITS = 11;
 static constexpr int RS_BINS = 1 << RS_BITS;
-static constexpr int RS_PASSES = 32 / RS_BITS;
-static constexpr int64_t SAMPLE = 65536;
+static constexpr int RS_PASSES = (32 + RS_BITS - 1) / RS_BITS;
+static constexpr int RS_PER = 8;                 // sample entries a thread
+static constexpr int64_t SAMPLE = RS_NT * RS_PER;
 
 // Order-preserving map float bits -> unsigned key (negative values reversed).
 __device__ __forceinline__ uint32_t fkey(float f) {
@@ -40,25 +48,19 @@ __device__ __forceinline__ float fkey_inv(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-struct SelectState {
-    unsigned long long hist[2][RS_BINS];
-    long long rank[2];          // rank still to find inside the current prefix
-    uint32_t prefix[2];         // key bits fixed so far (in the low bits)
-    int two;                    // 1 when two targets are tracked
-    int bits_done;              // leading key bits fixed so far (32: done)
-    int use_cand;               // histogram the candidate buffer (1) or all entries (0)
-    unsigned int arrived;       // blocks of the current launch that have finished
+struct SelectState {            // zeroed before the launch
+    unsigned bar;
+    int status;
     unsigned long long n_cand;  // entries found in [lo, hi]
     unsigned long long c_lo;    // entries found below lo
-    long long k1, k2;           // target ranks in the full data
+    unsigned long long hist[RS_PASSES][2][RS_BINS];
 };
 
-// The data a pass reads: a strided row-major view (rows x cols, leading dimension ld), or
-// the candidate buffer.  flat: the view is one contiguous run of rows * cols entries.
+// The data a pass reads: a strided row-major view (rows x cols, leading dimension ld).
+// flat: the view is one contiguous run of rows * cols entries.
 struct SelSrc {
     const float* x;
     int64_t rows, cols, ld;
-    const float* cand;
     int vec;   // 16-byte aligned rows (or run): float4 loads
     int flat;
 };
@@ -95,222 +97,243 @@ __device__ __forceinline__ void load_chunk(const SelSrc& src, int64_t t, int64_t
     }
 }
 
-// Block-wide digit pick (every thread of the block calls it; threads 0..RS_BINS-1 carry the
-// counts).  Thread d holds cnt = count[d]; the digit d with excl(d) <= rank < excl(d) +
-// count[d] lands in *s_digit and rank - excl(d) in *s_rank.  s_warp holds 8 words.
-__device__ __forceinline__ void block_pick(unsigned long long cnt, long long rank, unsigned long long* s_warp,
-                                           int* s_digit, long long* s_rank) {
+struct SelShared {
+    unsigned h[2][RS_BINS];
+    unsigned long long warp_sum[RS_NT / 32];
+    int digit, ok;
+    long long rank;
+    unsigned long long below[RS_NT / 32];
+};
+
+// Digit of the entry of rank `rank` in a histogram of RS_BINS counts (the whole block calls; bin
+// counts by `count`): the digit d with excl(d) <= rank < excl(d) + count(d), and rank - excl(d).
+template <typename Count>
+__device__ __forceinline__ void block_pick(Count count, long long* rank, uint32_t* digit, SelShared* sh) {
+    constexpr int PER = RS_BINS / RS_NT;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    unsigned long long incl = cnt;
+    unsigned long long c[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        c[k] = count(tid * PER + k);
+        sum += c[k];
+    }
+    unsigned long long incl = sum;
     for (int o = 1; o < 32; o <<= 1) {
         const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    if (tid < RS_BINS && lane == 31) s_warp[w] = incl;
+    __syncthreads();  // the shared words may still be read from the last pick
+    if (lane == 31) sh->warp_sum[w] = incl;
     if (tid == 0) {
-        *s_digit = RS_BINS - 1;  // kept only for an out-of-range rank, which cannot occur
-        *s_rank = rank;
+        sh->digit = RS_BINS - 1;  // kept only for an out-of-range rank, which cannot occur
+        sh->rank = *rank;
     }
     __syncthreads();
-    if (tid < RS_BINS) {
-        unsigned long long base = 0;
-        for (int k = 0; k < w; ++k) base += s_warp[k];
-        const long long excl = (long long)(base + incl - cnt);
-        if (cnt && rank >= excl && rank < excl + (long long)cnt) {
-            *s_digit = tid;
-            *s_rank = rank - excl;
+    unsigned long long before = 0;  // the warp totals before this one
+    {
+        const unsigned long long t = lane < w ? sh->warp_sum[lane] : 0ull;
+        before = t;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    }
+    long long excl = (long long)(before + incl - sum);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (c[k] && *rank >= excl && *rank < excl + (long long)c[k]) {
+            sh->digit = tid * PER + k;
+            sh->rank = *rank - excl;
         }
+        excl += (long long)c[k];
     }
     __syncthreads();
+    *digit = (uint32_t)sh->digit;
+    *rank = sh->rank;
 }
 
-// True in every thread of the last block of the launch to reach this point (the block's
-// global writes and atomics made before the call are then visible to it).
-__device__ __forceinline__ bool last_block(unsigned int* arrived) {
-    __shared__ int s_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = (atomicAdd(arrived, 1u) == gridDim.x - 1);
-    __syncthreads();
-    if (s_last) __threadfence();
-    return s_last;
-}
-
-__device__ __forceinline__ void state_init(SelectState* st, long long k1, long long k2) {
-    for (int t = threadIdx.x; t < 2 * RS_BINS; t += blockDim.x) (&st->hist[0][0])[t] = 0ull;
-    if (threadIdx.x == 0) {
-        st->rank[0] = k1;
-        st->rank[1] = k2;
-        st->prefix[0] = st->prefix[1] = 0u;
-        st->two = (k1 != k2);
-        st->bits_done = 0;
-        st->use_cand = 0;
-        st->arrived = 0u;
-        st->n_cand = 0ull;
-        st->c_lo = 0ull;
-        st->k1 = k1;
-        st->k2 = k2;
-    }
-}
-
-// Initialise the full-data state (ranks k1, k2) and, if given, the sample state.
-__global__ void rs_init(SelectState* st, long long k1, long long k2, SelectState* sst, long long s1, long long s2) {
-    state_init(st, k1, k2);
-    if (sst) state_init(sst, s1, s2);
-}
-
-// Fixed-stride sample: entry (n / s) * k of the row-major order, k < s.
-__global__ void rs_sample(SelSrc src, int64_t n, float* out) {
-    const int64_t step = n / SAMPLE;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < SAMPLE; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = step * k;
-        const int64_t r = t / src.cols, c = t - r * src.cols;
-        out[k] = __ldg(src.x + r * src.ld + c);
-    }
-}
-
-// Histogram of the next digit (the up to 8 key bits below the bits_done fixed ones) of the
-// keys whose fixed bits match; the last block picks the digits.  Reads the candidate buffer
-// when the state says so; does nothing once all 32 bits are fixed.  256 threads per block.
-__global__ void __launch_bounds__(256) rs_hist(SelSrc src, SelectState* st) {
-    const int hs = st->bits_done;
-    if (hs >= 32) return;
-    __shared__ unsigned int h[2][RS_BINS];
-    __shared__ unsigned long long s_warp[8];
-    __shared__ int s_digit;
-    __shared__ long long s_rank;
-    for (int t = threadIdx.x; t < 2 * RS_BINS; t += blockDim.x) (&h[0][0])[t] = 0u;
-    __syncthreads();
-    const int width = min(RS_BITS, 32 - hs);
-    const int shift = 32 - hs - width;
-    const uint32_t dmask = (1u << width) - 1u;
-    const uint32_t p0 = st->prefix[0], p1 = st->prefix[1];
-    const int two = st->two;
-    auto add = [&](float f, bool valid) {
+// The two targets of a radix select, the same in every thread.
+struct Targets {
+    long long rank[2];
+    uint32_t prefix[2];
+    int done;  // leading key bits fixed
+    __device__ __forceinline__ int width() const { return min(RS_BITS, 32 - done); }
+    __device__ __forceinline__ bool same() const { return prefix[0] == prefix[1]; }
+    // count key k into the histograms of its prefix (one histogram while the prefixes agree)
+    __device__ __forceinline__ void count(SelShared* sh, float f) const {
         const uint32_t k = fkey(f);
-        const uint32_t hi = hs ? (k >> (32 - hs)) : 0u;
-        const uint32_t d = (k >> shift) & dmask;
-        if (valid && hi == p0) atomicAdd(&h[0][d], 1u);
-        if (two && valid && hi == p1) atomicAdd(&h[1][d], 1u);
-    };
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // the candidate buffer is one aligned contiguous run of n_cand entries
-    const SelSrc in = st->use_cand ? SelSrc{src.cand, 1, (int64_t)st->n_cand, (int64_t)st->n_cand, nullptr, 1, 1} : src;
-    const int64_t n = n_chunks(in);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += stride) {
-        float v[4];
-        bool ok[4];
-        load_chunk(in, t, n, v, ok);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) add(v[e], ok[e]);
+        const uint32_t hi = done ? (k >> (32 - done)) : 0u;
+        const uint32_t d = (k >> (32 - done - width())) & ((1u << width()) - 1u);
+        if (hi == prefix[0]) atomicAdd(&sh->h[0][d], 1u);
+        else if (hi == prefix[1]) atomicAdd(&sh->h[1][d], 1u);
     }
+    template <typename Count>
+    __device__ __forceinline__ void pick(Count c, SelShared* sh) {
+        const int w = width(), other = same() ? 0 : 1;
+        uint32_t d0, d1;
+        block_pick([&](int b) { return c(0, b); }, &rank[0], &d0, sh);
+        block_pick([&](int b) { return c(other, b); }, &rank[1], &d1, sh);
+        prefix[0] = (prefix[0] << w) | d0;
+        prefix[1] = (prefix[1] << w) | d1;
+        done += w;
+    }
+};
+
+__device__ __forceinline__ void clear_hist(SelShared* sh) {
     __syncthreads();
-    for (int t = threadIdx.x; t < RS_BINS; t += blockDim.x) {
-        if (h[0][t]) atomicAdd(&st->hist[0][t], (unsigned long long)h[0][t]);
-        if (two && h[1][t]) atomicAdd(&st->hist[1][t], (unsigned long long)h[1][t]);
-    }
-    if (!last_block(&st->arrived)) return;
-    // last block: pick the digit of each target, clear the histograms for the next pass
-    for (int t = 0; t < 1 + two; ++t) {
-        const unsigned long long cnt = __ldcg(&st->hist[t][threadIdx.x]);
-        block_pick(cnt, st->rank[t], s_warp, &s_digit, &s_rank);
-        if (threadIdx.x == 0) {
-            st->rank[t] = s_rank;
-            st->prefix[t] = (st->prefix[t] << width) | (uint32_t)s_digit;
-        }
-        __syncthreads();
-    }
-    st->hist[0][threadIdx.x] = 0ull;
-    st->hist[1][threadIdx.x] = 0ull;
-    if (threadIdx.x == 0) {
-        st->bits_done = hs + width;
-        st->arrived = 0u;
-    }
+    for (int t = threadIdx.x; t < 2 * RS_BINS; t += RS_NT) (&sh->h[0][0])[t] = 0u;
+    __syncthreads();
 }
 
-// One pass over all entries: count those below lo, compact those in [lo, hi] (the first
-// `cap` of them are stored; the count keeps going so that an overflow is seen); lo and hi
-// are the values the sample state selected.  Each warp loads RS_UNROLL chunk groups before
-// testing them, stages its candidates in shared memory and reserves space in the buffer
-// once per GROUP or more of them.  The last block decides: candidates when they hold both
-// target ranks (then the leading bits that lo and hi share, which all candidates share too,
-// are fixed at once), else all entries.
 static constexpr int RS_UNROLL = 4;
-__global__ void __launch_bounds__(256) rs_count_compact(SelSrc src, const SelectState* sample_st, SelectState* st,
-                                                        float* cand, unsigned long long cap) {
-    constexpr int GROUP = 32 * RS_UNROLL * 4;  // entries a warp tests per iteration
-    constexpr int STAGE = 2 * GROUP;
-    __shared__ float s_stage[8][STAGE];
-    __shared__ unsigned long long s_below[8];
-    const uint32_t kl = sample_st->prefix[0], kh = sample_st->prefix[1];
-    const float lo = fkey_inv(kl), hi = fkey_inv(kh);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float* wb = s_stage[warp];
-    unsigned fill = 0;  // warp-uniform
-    unsigned long long below = 0;
-    auto flush = [&]() {
-        __syncwarp();
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&st->n_cand, (unsigned long long)fill);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        for (unsigned i = lane; i < fill; i += 32)
-            if (base + i < cap) cand[base + i] = wb[i];
-        __syncwarp();
-        fill = 0;
-    };
-    const int64_t n = n_chunks(src);
-    const int64_t gwarp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    // whole warps walk the chunk space together (the compaction uses warp ballots)
-    for (int64_t t0 = gwarp * 32 * RS_UNROLL; t0 < n; t0 += nwarps * 32 * RS_UNROLL) {
-        float v[RS_UNROLL][4];
-        bool ok[RS_UNROLL][4];
+static constexpr int RS_GROUP = 32 * RS_UNROLL * 4;  // entries a warp tests per iteration
+static constexpr int RS_STAGE = RS_GROUP + 256;      // entries a warp stages before it writes them out
+static constexpr size_t RS_SMEM = sizeof(SelShared) + sizeof(float) * (RS_NT / 32) * RS_STAGE;
+
+// out[0] = median, out[1] = 0; out[1] stays 1 when a wait gave up.
+__global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, long long k1, long long k2, int bracket,
+                                                      long long s1, long long s2, SelectState* st, float* cand,
+                                                      unsigned long long cap, long long spin, double* out) {
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    SelShared* sh = reinterpret_cast<SelShared*>(rs_smem);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned nb = gridDim.x;
+    unsigned gen = 0;
+    if (blockIdx.x == 0 && tid == 0) out[1] = 1.0;
+// leaves the kernel when the wait gave up
+#define RS_BARRIER()                                                                                       \
+    do {                                                                                                   \
+        if (!grid_barrier_named(&st->bar, nb * ++gen, &st->status, spin, 1, RS_NT, &sh->ok)) return;      \
+    } while (0)
+    Targets T;
+    T.rank[0] = k1;
+    T.rank[1] = k2;
+    T.prefix[0] = T.prefix[1] = 0u;
+    T.done = 0;
+    bool use_cand = false;
+    const int64_t nch = n_chunks(src);
+    if (bracket) {
+        // ---- bracket from a sample, by every CTA alike -------------------------------------
+        Targets B;
+        B.rank[0] = s1;
+        B.rank[1] = s2;
+        B.prefix[0] = B.prefix[1] = 0u;
+        B.done = 0;
+        float v[RS_PER];
+        const uint64_t step = (uint64_t)n / SAMPLE;
 #pragma unroll
-        for (int u = 0; u < RS_UNROLL; ++u) load_chunk(src, t0 + 32 * u + lane, n, v[u], ok[u]);
-#pragma unroll
-        for (int u = 0; u < RS_UNROLL; ++u) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                below += (ok[u][e] && v[u][e] < lo) ? 1ull : 0ull;
-                const bool in = ok[u][e] && v[u][e] >= lo && v[u][e] <= hi;
-                const unsigned m = __ballot_sync(0xffffffffu, in);
-                if (in) wb[fill + __popc(m & ((1u << lane) - 1u))] = v[u][e];
-                fill += __popc(m);
+        for (int e = 0; e < RS_PER; ++e) {
+            const uint32_t k = tid + RS_NT * e;
+            // the place inside the k-th part: hashed, so that it does not follow the rows
+            const uint64_t t = step * k + (((uint64_t)(k * 2654435761u) * step) >> 32);
+            if (src.flat) {
+                v[e] = __ldg(src.x + t);
+            } else {
+                const uint64_t r = t / (uint64_t)src.cols;
+                v[e] = __ldg(src.x + r * src.ld + (t - r * src.cols));
             }
         }
-        if (fill >= STAGE - GROUP) flush();  // keep room for one more iteration
+        for (int pass = 0; pass < RS_PASSES; ++pass) {
+            clear_hist(sh);
+#pragma unroll
+            for (int e = 0; e < RS_PER; ++e) B.count(sh, v[e]);
+            __syncthreads();
+            B.pick([&](int t, int b) { return (unsigned long long)sh->h[t][b]; }, sh);
+        }
+        const uint32_t kl = B.prefix[0], kh = B.prefix[1];
+        // ---- count those below, compact those inside ------------------------------------------
+        // Each warp loads RS_UNROLL chunk groups before testing them, stages its candidates in
+        // shared memory and reserves room in the buffer once per 256 or more of them.
+        float* wb = reinterpret_cast<float*>(rs_smem + sizeof(SelShared)) + warp * RS_STAGE;
+        unsigned fill = 0;  // warp-uniform
+        unsigned long long below = 0;
+        auto flush = [&]() {
+            __syncwarp();
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(&st->n_cand, (unsigned long long)fill);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            for (unsigned i = lane; i < fill; i += 32)
+                if (base + i < cap) cand[base + i] = wb[i];
+            __syncwarp();
+            fill = 0;
+        };
+        const int64_t gwarp = (int64_t)blockIdx.x * (RS_NT / 32) + warp, nwarps = (int64_t)nb * (RS_NT / 32);
+        // whole warps walk the chunk space together (the compaction uses warp ballots)
+        for (int64_t t0 = gwarp * 32 * RS_UNROLL; t0 < nch; t0 += nwarps * 32 * RS_UNROLL) {
+            float x[RS_UNROLL][4];
+            bool ok[RS_UNROLL][4];
+#pragma unroll
+            for (int u = 0; u < RS_UNROLL; ++u) load_chunk(src, t0 + 32 * u + lane, nch, x[u], ok[u]);
+            unsigned lt = 0;
+#pragma unroll
+            for (int u = 0; u < RS_UNROLL; ++u) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t k = fkey(x[u][e]);
+                    lt += ok[u][e] && k < kl;
+                    const bool in = ok[u][e] && k - kl <= kh - kl;
+                    const unsigned m = __ballot_sync(0xffffffffu, in);
+                    if (in) wb[fill + __popc(m & ((1u << lane) - 1u))] = x[u][e];
+                    fill += __popc(m);
+                }
+            }
+            below += lt;
+            if (fill > RS_STAGE - RS_GROUP) flush();  // keep room for one more iteration
+        }
+        if (fill) flush();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+        if (lane == 0) sh->below[warp] = below;
+        __syncthreads();
+        if (tid == 0) {
+            unsigned long long b = 0;
+            for (int w = 0; w < RS_NT / 32; ++w) b += sh->below[w];
+            atomicAdd(&st->c_lo, b);
+        }
+        RS_BARRIER();
+        const long long c_lo = (long long)__ldcg(&st->c_lo), nc = (long long)__ldcg(&st->n_cand);
+        const long long a = k1 - c_lo, b = k2 - c_lo;
+        use_cand = nc <= (long long)cap && a >= 0 && a < nc && b >= 0 && b < nc;
+        if (use_cand) {
+            src = SelSrc{cand, 1, nc, nc, 1, 1};  // an aligned contiguous run
+            T.rank[0] = a;
+            T.rank[1] = b;
+            T.done = __clz((int)(kl ^ kh));  // 32 when lo == hi
+            T.prefix[0] = T.prefix[1] = T.done == 0 ? 0u : (T.done == 32 ? kl : (kl >> (32 - T.done)));
+        }
     }
-    if (fill) flush();
-    for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
-    if (lane == 0) s_below[warp] = below;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long b = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += s_below[w];
-        atomicAdd(&st->c_lo, b);
+    // ---- radix select over the candidates, or over all entries ----------------------------------
+    const int64_t m = n_chunks(src);
+    for (int pass = 0; T.done < 32; ++pass) {
+        clear_hist(sh);
+        for (int64_t t = (int64_t)blockIdx.x * RS_NT + tid; t < m; t += (int64_t)nb * RS_NT) {
+            float x[4];
+            bool ok[4];
+            if (use_cand) {  // written by other SMs in this launch: not through the read-only path
+                const int64_t left = src.cols - 4 * t;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    ok[e] = e < left;
+                    x[e] = ok[e] ? __ldcg(cand + 4 * t + e) : 0.f;
+                }
+            } else {
+                load_chunk(src, t, m, x, ok);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (ok[e]) T.count(sh, x[e]);
+        }
+        __syncthreads();
+        for (int t = tid; t < 2 * RS_BINS; t += RS_NT) {
+            const unsigned c = (&sh->h[0][0])[t];
+            if (c) atomicAdd(&st->hist[pass][0][0] + t, (unsigned long long)c);
+        }
+        RS_BARRIER();
+        T.pick([&](int t, int b) { return __ldcg(&st->hist[pass][t][b]); }, sh);
     }
-    if (!last_block(&st->arrived)) return;
-    if (threadIdx.x == 0) {
-        const long long c_lo = (long long)__ldcg(&st->c_lo);
-        const long long nc = (long long)__ldcg(&st->n_cand);
-        const long long a = st->k1 - c_lo, b = st->k2 - c_lo;
-        const int ok = nc <= (long long)cap && a >= 0 && a < nc && b >= 0 && b < nc;
-        st->use_cand = ok;
-        st->rank[0] = ok ? a : st->k1;
-        st->rank[1] = ok ? b : st->k2;
-        const int common = ok ? __clz((int)(kl ^ kh)) : 0;  // 32 when lo == hi
-        st->prefix[0] = st->prefix[1] = common == 0 ? 0u : (common == 32 ? kl : (kl >> (32 - common)));
-        st->bits_done = common;
-        st->arrived = 0u;
+    if (blockIdx.x == 0 && tid == 0) {
+        out[0] = 0.5 * ((double)fkey_inv(T.prefix[0]) + (double)fkey_inv(T.prefix[1]));
+        out[1] = 0.0;
     }
-}
-
-__global__ void rs_finish(const SelectState* st, double* out) {
-    if (threadIdx.x == 0) {
-        const double a = (double)fkey_inv(st->prefix[0]);
-        const double b = st->two ? (double)fkey_inv(st->prefix[1]) : a;
-        *out = 0.5 * (a + b);
-    }
+#undef RS_BARRIER
 }
 
 ot_status launch_median(ot_assoc_ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t ld, double* out_dev,
@@ -320,48 +343,38 @@ ot_status launch_median(ot_assoc_ctx* ctx, const float* x, int64_t rows, int64_t
     const long long k1 = (n - 1) / 2, k2 = n / 2;  // equal for odd n
     const int flat = (rows == 1 || ld == cols);
     const int vec = !((uintptr_t)x & 15u) && (flat || ld % 4 == 0);
-    const SelSrc src0{x, rows, cols, ld, nullptr, vec, flat};
-    const int64_t nch = n_chunks(src0);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nch + 255) / 256, 8LL * ctx->num_sms));
-    const bool bracket = n >= 16 * SAMPLE;  // below that, four passes over the data cost little
-    // the bracket spans about 2.3% of the entries; more than n/16 means heavy ties
+    const SelSrc src{x, rows, cols, ld, vec, flat};
+    const int64_t nch = n_chunks(src);
+    const int bracket = n >= (1 << 20);  // below that, three passes over the data cost little
+    // the bracket spans about 5% of the entries; more than n/16 means heavy ties
     const unsigned long long cap = bracket ? (unsigned long long)(n / 16) : 0ull;
-    const size_t off_sst = (size_t)round_up(sizeof(SelectState), 256);
-    const size_t off_sample = off_sst + (size_t)round_up(sizeof(SelectState), 256);
-    const size_t off_cand = off_sample + sizeof(float) * (size_t)SAMPLE;
-    const size_t bytes = bracket ? off_cand + sizeof(float) * (size_t)cap : sizeof(SelectState);
-    char* ws = (char*)scratch(ctx, SLOT_SELECT, bytes, &st);
+    const size_t off_cand = (size_t)round_up(sizeof(SelectState), 256);
+    char* ws = (char*)scratch(ctx, SLOT_SELECT, off_cand + sizeof(float) * (size_t)cap, &st);
     if (st) return st;
     SelectState* ss = (SelectState*)ws;
-    SelSrc src = src0;
-    int launches = 0;
-    int hist_grid = grid;
-    if (bracket) {
-        SelectState* sst = (SelectState*)(ws + off_sst);
-        float* sample = (float*)(ws + off_sample);
-        float* cand = (float*)(ws + off_cand);
-        const double sd = 0.5 * std::sqrt((double)SAMPLE);
-        const long long slo = (long long)(SAMPLE / 2 - 6.0 * sd);
-        const long long shi = (long long)(SAMPLE / 2 + 6.0 * sd);
-        rs_init<<<1, 256, 0, s>>>(ss, k1, k2, sst, slo, shi);
-        rs_sample<<<(int)(SAMPLE / 256), 256, 0, s>>>(src, n, sample);
-        const SelSrc ssrc{sample, 1, SAMPLE, SAMPLE, nullptr, 1, 1};
-        for (int pass = 0; pass < RS_PASSES; ++pass) rs_hist<<<(int)(SAMPLE / 1024), 256, 0, s>>>(ssrc, sst);
-        rs_count_compact<<<grid, 256, 0, s>>>(src, sst, ss, cand, cap);
-        src.cand = cand;
-        // candidates are at most n/16 entries; the rare full-data fallback runs on this grid too
-        hist_grid = std::max(1, std::min(grid, 2 * ctx->num_sms));
-        launches += 3 + RS_PASSES;
-    } else {
-        rs_init<<<1, 256, 0, s>>>(ss, k1, k2, nullptr, 0, 0);
-        ++launches;
+    float* cand = (float*)(ws + off_cand);
+    const double sd = 0.5 * std::sqrt((double)SAMPLE);
+    const long long s1 = (long long)(SAMPLE / 2 - 4.5 * sd), s2 = (long long)(SAMPLE / 2 + 4.5 * sd);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nch + RS_NT - 1) / RS_NT, ctx->num_sms));
+    if (allow_max_dynamic_smem((const void*)rs_select, RS_SMEM) != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(ctx, OT_ECUDA, "median kernel: %zu bytes of shared memory refused", RS_SMEM);
     }
-    for (int pass = 0; pass < RS_PASSES; ++pass) rs_hist<<<hist_grid, 256, 0, s>>>(src, ss);
-    rs_finish<<<1, 32, 0, s>>>(ss, out_dev);
-    launches += 1 + RS_PASSES;
-    ctx->launches += launches;
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelectState), s);
+    if (e != cudaSuccess) return cuda_error(ctx, e, "median memset");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(RS_NT);
+    cfg.dynamicSmemBytes = RS_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, rs_select, src, n, k1, k2, bracket, s1, s2, ss, cand, cap, 1LL << 24, out_dev);
     if (e != cudaSuccess) return cuda_error(ctx, e, "median launch");
+    ctx->launches += 1;
     return OT_OK;
 }
 

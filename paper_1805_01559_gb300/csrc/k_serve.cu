@@ -615,15 +615,16 @@ ot_status ot_assoc_build_cost_mobile(ot_assoc_ctx* ctx, double* dev_xy, double* 
     struct {
         int bad;
         int pad;
-        double med;
+        double med[2];
     }* h = (decltype(h))host_staging(ctx, 64, &st);
     if (st) return st;
     e = cudaMemcpyAsync(&h->bad, dstat, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h->med, dmed, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->med, dmed, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "mobile cost");
     if (h->bad != DEV_OK) return set_error(ctx, OT_EINVAL, "some rate is not finite and > 0");
-    *eps_out = eps_rel * h->med;
+    if (h->med[1] != 0.0) return set_error(ctx, OT_ETIMEOUT, "median: a device-side wait exceeded its spin limit");
+    *eps_out = eps_rel * h->med[0];
     return OT_OK;
 }
 
@@ -852,14 +853,19 @@ ot_status ot_assoc_server_add_cell(ot_assoc_server* s, const ot_assoc_cell_desc*
                 return st;
             }
         }
-        double med = 0.0;
+        double medv[2] = {0.0, 0.0};
         int hs = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&med, dmed, sizeof(double), cudaMemcpyDeviceToHost, s->run_stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(medv, dmed, sizeof(medv), cudaMemcpyDeviceToHost, s->run_stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, dstat, sizeof(int), cudaMemcpyDeviceToHost, s->run_stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->run_stream);
         if (e != cudaSuccess) {
             sv_free_cell(s, c);
             return cuda_error(ctx, e, "first instance");
+        }
+        const double med = medv[0];
+        if (medv[1] != 0.0) {
+            sv_free_cell(s, c);
+            return set_error(ctx, OT_ETIMEOUT, "median: a device-side wait exceeded its spin limit");
         }
         if (hs != DEV_OK || !(med > 0.0) || !std::isfinite(med)) {
             sv_free_cell(s, c);

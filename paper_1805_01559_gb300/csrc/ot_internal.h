@@ -160,7 +160,8 @@ ot_status launch_cost(ot_assoc_ctx* ctx, const float* R, int64_t ld_r, int64_t I
                       float* C, int64_t ld_c, bool pad_inf, unsigned long long* bad_dev,
                       cudaStream_t s);
 // Median of the first n entries of a strided matrix view (rows x cols, ld) of floats; writes
-// the result (double) to *out_dev.  Requires no NaN.
+// the result (double) to out_dev[0] and 0 to out_dev[1], which is 1 when a wait of the launch
+// gave up.  Requires no NaN.
 ot_status launch_median(ot_assoc_ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t ld,
                         double* out_dev, cudaStream_t s);
 // Batched ragged solve (k_batch.cu).

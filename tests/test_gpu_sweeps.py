@@ -116,3 +116,27 @@ def test_group_with_idle_ctas(kind):
         c.solve_batched(inst)
         for x in inst:
             assert torch.equal(x.f, one.f) and torch.equal(x.g, one.g)
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (1, 3), (3, 5), (1000, 50), (1024, 1023), (1024, 1024), (1025, 1026), (3000, 801)])
+@pytest.mark.parametrize("kind", ["lognormal", "signs", "two_values", "outside"])
+def test_median_strided_edges(ctx, shape, kind):
+    """Median of a padded view on both sides of 2^20 entries, exact: values of both signs with
+    zeros of both signs, two values only, and a middle that nearly no sampled entry is near."""
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 31 + J))
+    x = rng.lognormal(0.0, 2.0, (I, J)).astype(np.float32)
+    if kind == "signs":
+        x *= rng.choice(np.array([-1.0, 0.0, -0.0, 1.0], np.float32), (I, J))
+    elif kind == "two_values":
+        x = np.where(rng.random((I, J)) < 0.5, np.float32(1.0), np.float32(2.0)).astype(np.float32)
+    elif kind == "outside":
+        x.reshape(-1)[: (I * J) // 2] = 1e-30
+    pad = torch.full((I, J + 3), -7.0, dtype=torch.float32, device="cuda")
+    pad[:, :J] = torch.from_numpy(x).cuda()
+    if I > 1:
+        R = torch.from_numpy(np.abs(x) + np.float32(1.0)).cuda()
+        C, eps = ctx.build_cost(R, 1.0, eps_rel=1.0, C_out=pad[:, :J])
+        assert eps == oracle.median(C.cpu().numpy().astype(np.float64))
+    flat = torch.from_numpy(x.reshape(-1)).cuda()
+    assert ctx.median_f32(flat) == oracle.median(x.astype(np.float64))
