@@ -46,6 +46,7 @@ struct LoopState {
 //   [4 Jp, 4.5 Jp)  fixed-point shift S_j of column j (int)
 //   then 2 rows of Jp + 4 64-bit words: per-column fixed-point totals of the sweeps' column
 //   partials and their row residuals (word Jp); sweep s adds into row s mod 2.
+//   then Jp FP32 pairs: G^0, later G^1, as the sweeps hold them.
 // The totals are sums of integers, the same in any order, so every CTA reads the same column
 // sums whatever the number of CTAs or the order in which partitions arrive.
 //
@@ -59,12 +60,21 @@ static constexpr int FX_BITS = 40;   // a column total of q^_j is about 2^40 uni
 static constexpr int FX_TOP = 48;    // partials (and totals) from 2^48 on go to the exact path
 static constexpr int FX_ERR = 50;    // row residuals in units of 2^-50
 static constexpr int FX_COUNT = 56;  // bit position of the partition count
-__host__ __device__ constexpr size_t gstate_words(int Jp) { return (size_t)Jp * 13 / 2 + 8; }
+__host__ __device__ constexpr size_t gstate_words(int Jp) { return (size_t)Jp * 15 / 2 + 8; }
 __host__ __device__ constexpr size_t gstate_bytes(int Jp) { return 8 * gstate_words(Jp); }
 __device__ __forceinline__ float2* gs_lq2(double* G, int Jp) { return reinterpret_cast<float2*>(G + 3 * (size_t)Jp); }
 __device__ __forceinline__ int* gs_sx(double* G, int Jp) { return reinterpret_cast<int*>(G + 4 * (size_t)Jp); }
 __device__ __forceinline__ unsigned long long* gs_acc(double* G, int Jp) {
     return reinterpret_cast<unsigned long long*>(G + 4 * (size_t)Jp + Jp / 2);
+}
+
+__device__ __forceinline__ float2* gs_pairs(double* G, int Jp) {
+    return reinterpret_cast<float2*>(G + (size_t)Jp * 13 / 2 + 8);
+}
+// An FP64 value as an FP32 pair, to about 2^-48 relative.
+__device__ __forceinline__ float2 split_pair(double x) {
+    const float hi = (float)x;
+    return make_float2(hi, (float)(x - (double)hi));
 }
 
 template <int TW, int VPT>
@@ -164,6 +174,17 @@ __device__ __forceinline__ void load_G_smem(const double* __restrict__ G, int J,
         const float hi = (float)x;
         Gs[j] = hi;
         Gs[Jp + j] = (float)(x - (double)hi);
+    }
+}
+
+// The same from pairs formed elsewhere (one thread a column of the whole group, instead of
+// FP64 conversions of every column in every CTA).
+__device__ __forceinline__ void load_G_pairs(const float2* __restrict__ pairs, int J, int Jp, float* Gs, int tid,
+                                             int nthreads) {
+    for (int j = tid; j < Jp; j += nthreads) {
+        const float2 x = j < J ? __ldcg(pairs + j) : make_float2(0.f, 0.f);
+        Gs[j] = x.x;
+        Gs[Jp + j] = x.y;
     }
 }
 
@@ -980,6 +1001,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     } while (0)
 
     // ---- setup: sums of p (per partition) and q (every CTA), checks, starting G ----------
+    // An SM takes an FP64 warp instruction about every 16 cycles, so what all warps do alike in
+    // FP64 adds up: the totals below, formed by all 15 of them, took 17,000 cycles, log2 q^ by
+    // the warps of a few CTAs 11,000.  Sums are formed by the warps that hold terms (an absent
+    // term is a zero), combined by one warp, and columns are dealt to the CTAs one warp each.
+    const int swarp = warp * nb + b, nw = nb * NCW;  // this warp among the group's, CTA by CTA
     {
         int bad = 0;
         for (int v = v0; v < v1; ++v) {
@@ -991,21 +1017,23 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 sp += (double)x;
                 Ps[r] = x;
             }
-            sp = warp_sum(sp);
-            if (lane == 0) sh_sum[warp][0] = sp;
+            if (warp * 32 < e - a) {
+                sp = warp_sum(sp);
+                if (lane == 0) sh_sum[warp][0] = sp;
+            }
             bar_named(CONS_BAR, NC);
             if (tid == 0) {
                 double t = 0.0;
-                for (int w = 0; w < NCW; ++w) t += sh_sum[w][0];
+                for (int w = 0; w < NCW && w * 32 < e - a; ++w) t += sh_sum[w][0];
                 P.errpart[v] = t;
             }
             bar_named(CONS_BAR, NC);
         }
-        const int gw = b * NCW + warp, nw = nb * NCW;
-        for (int j = gw * 32 + lane; j < J; j += nw * 32) {
+        for (int j = swarp * 32 + lane; j < J; j += nw * 32) {
             const double g0 = P.g_warm ? P.g_warm[j] * P.k : 0.0;
             bad |= !isfinite(g0);
             P.G[j] = g0;
+            gs_pairs(P.G, Jp)[j] = split_pair(g0);
         }
         if (b == 0 && tid == 0 && P.input_bad && *P.input_bad) bad = 1;
         if (bad) atomicOr(&s_bad, 1);
@@ -1013,19 +1041,24 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         if (tid == 0 && s_bad) atomicCAS(status, DEV_OK, DEV_EINVAL);
     }
     OTA_BARRIER_CHECK();
-    double sp = 0.0, sq = 0.0;
+    double inv_sq;
+    float inv_sp_f;
     {
         // every CTA forms the same totals in the same order
         double a = 0.0, c = 0.0;
         int badq = 0;
-        for (int bb = tid; bb < V; bb += NC) a += P.errpart[bb];
-        for (int j = tid; j < J; j += NC) {
-            const float x = __ldcg(P.q + j);
-            badq |= !(x > 0.0f) || !isfinite(x);
-            c += (double)x;
+        if (warp * 32 < V) {
+            for (int bb = tid; bb < V; bb += NC) a += P.errpart[bb];
+            a = warp_sum(a);
         }
-        a = warp_sum(a);
-        c = warp_sum(c);
+        if (warp * 32 < J) {
+            for (int j = tid; j < J; j += NC) {
+                const float x = __ldcg(P.q + j);
+                badq |= !(x > 0.0f) || !isfinite(x);
+                c += (double)x;
+            }
+            c = warp_sum(c);
+        }
         if (tid == 0) s_bad = 0;
         bar_named(CONS_BAR, NC);
         if (lane == 0) {
@@ -1034,43 +1067,51 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         }
         if (badq) atomicOr(&s_bad, 1);
         bar_named(CONS_BAR, NC);
-        for (int w = 0; w < NCW; ++w) {
-            sp += sh_sum[w][0];
-            sq += sh_sum[w][1];
+        if (warp == 0) {  // lane 0 the sum of p, lane 1 of q
+            double t = 0.0;
+            for (int w = 0; w < NCW; ++w) t += sh_sum[w][lane & 1];
+            const double inv = 1.0 / t;
+            const double sp = __shfl_sync(0xffffffffu, t, 0), sq = __shfl_sync(0xffffffffu, t, 1);
+            const double inv_p = __shfl_sync(0xffffffffu, inv, 0), inv_q = __shfl_sync(0xffffffffu, inv, 1);
+            __syncwarp();
+            if (lane == 0) {
+                sh->s_dec = s_bad || !(fabs(sp - sq) <= 1e-5 * sp);
+                sh_sum[0][0] = inv_q;
+                sh_sum[0][1] = inv_p;
+                if (b == 0 && !sh->s_dec) {
+                    P.sc->sp = sp;
+                    P.sc->sq = sq;
+                    P.sc->inv_sp = inv_p;
+                    P.sc->inv_sq = inv_q;
+                    P.sc->inv_sp_f = (float)inv_p;
+                    P.sc->status = DEV_OK;
+                }
+            }
         }
-        if (s_bad || !(fabs(sp - sq) <= 1e-5 * sp)) {
+        bar_named(CONS_BAR, NC);
+        if (sh->s_dec) {
             if (b == 0 && tid == 0) atomicCAS(status, DEV_OK, DEV_EINVAL);
             if (tid == 0) s_stop = 1;
             return false;  // the same decision in every CTA
         }
-        if (b == 0 && tid == 0) {
-            P.sc->sp = sp;
-            P.sc->sq = sq;
-            P.sc->inv_sp = 1.0 / sp;
-            P.sc->inv_sq = 1.0 / sq;
-            P.sc->inv_sp_f = (float)(1.0 / sp);
-            P.sc->status = DEV_OK;
-        }
+        inv_sq = sh_sum[0][0];
+        inv_sp_f = (float)sh_sum[0][1];
     }
-    const double inv_sq = 1.0 / sq;
     double* LQ = P.G + 2 * Jp;  // log2 q^_j, formed once here (read after the next grid barrier)
     float2* LQ2 = gs_lq2(P.G, Jp);
     int* SX = gs_sx(P.G, Jp);
     unsigned long long* ACC = gs_acc(P.G, Jp);
     {
-        const int gw = b * NCW + warp, nw = nb * NCW;
-        for (int j = gw * 32 + lane; j < J; j += nw * 32) {
+        for (int j = swarp * 32 + lane; j < J; j += nw * 32) {
             const double lq = log2((double)__ldcg(P.q + j) * inv_sq);
             LQ[j] = lq;
-            const float hi = (float)lq;
-            LQ2[j] = make_float2(hi, (float)(lq - (double)hi));
+            LQ2[j] = split_pair(lq);
             // the total of column j is about 2^FX_BITS when its sum is q^_j; shifts that the
             // FP32 scale cannot carry send the column to the exact path (shift 0 = "never")
             const int sx = FX_BITS - (int)floor(lq);
             SX[j] = sx <= 126 ? sx : 0;
         }
-        for (int t = (b * NCW + warp) * 32 + lane; t < 2 * (Jp + 4); t += nw * 32) ACC[t] = 0ull;
-        const float inv_sp_f = (float)(1.0 / sp);
+        for (int t = swarp * 32 + lane; t < 2 * (Jp + 4); t += nw * 32) ACC[t] = 0ull;
         for (int r = tid; r < nrow; r += NC) Ps[r] *= inv_sp_f;  // p^_i
         bar_named(CONS_BAR, NC);
     }
@@ -1085,7 +1126,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         if (tid == 0) s_stop = 1;
         return true;
     }
-    load_G_smem(P.G, J, Jp, Gs, tid, NC);
+    load_G_pairs(gs_pairs(P.G, Jp), J, Jp, Gs, tid, NC);
     bar_named(CONS_BAR, NC);
     int par = 0;
 
@@ -1170,8 +1211,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         OTA_BARRIER();
         // G^1_j = G^0_j + log2 q^_j - log2(column sum of pi^(1/2)), one warp per column
         {
-            const int gw = b * NCW + warp, nw = nb * NCW;
-            for (int j = gw; j < J; j += nw) {
+            for (int j = swarp; j < J; j += nw) {
                 float2 sum = make_float2(0.f, 0.f);
                 for (int bb = lane; bb < V; bb += 32) sum = df_add(sum, P.colpart[(int64_t)bb * Jp + j]);
                 sum = warp_sum_df(sum);
@@ -1180,7 +1220,9 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                         atomicOr(flag1, 1ull);
                     } else {
                         const float2 ls = df_log2(sum);
-                        P.G[Jp + j] = P.G[j] + LQ[j] - (((double)ls.x - 64.0) + (double)ls.y);
+                        const double g1 = P.G[j] + LQ[j] - (((double)ls.x - 64.0) + (double)ls.y);
+                        P.G[Jp + j] = g1;
+                        gs_pairs(P.G, Jp)[j] = split_pair(g1);
                     }
                 }
             }
@@ -1188,7 +1230,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         OTA_BARRIER_CHECK();
         exact1 = __ldcg(flag1) != 0ull;
         if (!exact1) {
-            load_G_smem(P.G + Jp, J, Jp, Gs, tid, NC);
+            load_G_pairs(gs_pairs(P.G, Jp), J, Jp, Gs, tid, NC);
             bar_named(CONS_BAR, NC);
         }
     }
@@ -1349,8 +1391,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         OTA_BARRIER();
         // G^1_j = G^0_j + log2 q^_j - log2(column sum of pi^(1/2)), one warp per column
         {
-            const int gw = b * NCW + warp, nw = nb * NCW;
-            for (int j = gw; j < J; j += nw) {
+            for (int j = swarp; j < J; j += nw) {
                 float mm = -INFINITY;
                 for (int bb = lane; bb < V; bb += 32) mm = fmaxf(mm, part2[(int64_t)bb * Jp + j].x);
                 mm = warp_max(mm);
