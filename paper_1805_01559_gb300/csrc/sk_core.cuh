@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <float.h>
 #include <math.h>
 
 #include <type_traits>
@@ -555,15 +556,125 @@ __device__ __forceinline__ void cta_col_sum(float* comb, const float4 (&acc)[VPT
     bar_named(CONS_BAR, NC);
 }
 
+// ---- packed FP32 pairs: one instruction for two columns (fma/add .f32x2), each half rounded
+// exactly as the scalar operation rounds it. ------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Column potentials in tensor memory: the eight words of chunk v (four high parts, four low
+// parts) of a lane at columns 8 v .. 8 v + 7 of its warp's quarter.  Lane positions repeat
+// every TW warps, so one copy per quarter serves every warp of the CTA (two for teams of 8).
+// The sweep reads G (eight bytes a column) once per row: from shared memory that was two thirds
+// of its shared-memory wavefronts (84 a row of 800 columns, with 25 more for the copy that
+// fills the ring), the busiest unit of the sweep.  Out of tensor memory the sweep of a
+// 50,000 x 800 solve takes 41,000 cycles a CTA instead of 46,600, and the whole solve 0.98 ms
+// instead of 1.00 (1.04 before the packed arithmetic); 100,000 x 1,536: 2.50 ms against 3.03.
+template <int TW, int VPT>
+constexpr int tmem_cols() {
+    constexpr int n = 8 * VPT * (TW == 8 ? 2 : 1);
+    return n <= 32 ? 32 : (n <= 64 ? 64 : 128);
+}
+template <int TW, int VPT>
+__device__ __forceinline__ uint32_t tmem_G(uint32_t base, const Team<TW>& tm) {
+    const uint32_t warp = threadIdx.x >> 5;
+    return base + ((warp & 3u) << 21) + (TW == 8 ? (uint32_t)(tm.wit >> 2) * (8 * VPT) : 0u);
+}
+// Copy G from shared memory to tensor memory (all consumer warps call; G complete in Gs before,
+// visible to every consumer warp after).
+template <int TW, int VPT>
+__device__ __forceinline__ void G_to_tmem(uint32_t base, const float* Gs, int Jp, const Team<TW>& tm) {
+    constexpr int WRITERS = TW == 8 ? 8 : 4, TT = 32 * TW;
+    if ((threadIdx.x >> 5) < WRITERS) {
+        const uint32_t a = tmem_G<TW, VPT>(base, tm);
+        tmem_fence_after();
+#pragma unroll
+        for (int v = 0; v < VPT; ++v) {
+            const int col = 4 * (tm.tl + TT * v);
+            float4 hi = make_float4(0.f, 0.f, 0.f, 0.f), lo = hi;
+            if (col < Jp) {
+                hi = *reinterpret_cast<const float4*>(Gs + col);
+                lo = *reinterpret_cast<const float4*>(Gs + Jp + col);
+            }
+            __syncwarp();
+            tmem_st8(a + 8 * v, hi, lo);
+        }
+        tmem_wait_st();
+        tmem_fence_before();
+    }
+    bar_named(CONS_BAR, Cons<TW>::NCW * 32);
+    tmem_fence_after();
+}
+
+// A lane's chunk of G as two packed pairs of high and of low parts: from tensor memory (TM), or
+// from shared memory.  The whole warp calls it, converged.
+template <bool TM>
+__device__ __forceinline__ void load_G_chunk(uint32_t tG, int v, const float* Gs, int Jp, int col, f32x2 (&gh)[2],
+                                             f32x2 (&gl)[2]) {
+    if constexpr (TM) {
+        uint32_t w[8];
+        tmem_ld8(tG + 8 * v, w);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            gh[h] = pack2(__uint_as_float(w[2 * h]), __uint_as_float(w[2 * h + 1]));
+            gl[h] = pack2(__uint_as_float(w[4 + 2 * h]), __uint_as_float(w[5 + 2 * h]));
+        }
+    } else {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(Gs + col);
+        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(Gs + Jp + col);
+        gh[0] = a.x;
+        gh[1] = a.y;
+        gl[0] = b.x;
+        gl[1] = b.y;
+    }
+}
+// A lane's chunk of a row of C as two packed pairs, formed from coordinates when EUC.
+template <bool EUC>
+__device__ __forceinline__ void load_C_chunk(const float* row, float2 dxy, const float* rxs, int Jp, int J, int col,
+                                             f32x2 (&c)[2]) {
+    if constexpr (EUC) {
+        const float4 e = euclid_chunk(dxy, rxs, rxs + Jp, col, J);
+        c[0] = pack2(e.x, e.y);
+        c[1] = pack2(e.z, e.w);
+    } else {
+        const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(row + col);
+        c[0] = e.x;
+        c[1] = e.y;
+    }
+}
+
 // Finalize sweep of the consumer warps, run right after the loop stops: the producer has
 // already streamed the next pass over the CTA's rows into the ring, so this is one more
 // sweep at streaming speed.  Plan of the returned potentials F' (Fold) and G (Gs, still the
-// returned plan's column potentials): t_ij = 2^(F'_i + G_j - k C_ij).  Each team keeps FP32
+// returned plan's column potentials, also in tensor memory when TM): t_ij = 2^(F'_i + G_j - k C_ij).  Each team keeps FP32
 // column sums of p^ t and p^ C t over at most FIN_ROWS rows, then the CTA adds the teams'
 // sums (in team order) into the partition's FP64 partials P.fpart[v]; the row residual
 // sum_i p^_i |sum_j t_ij - 1| uses error-free row sums.
 static constexpr int FIN_ROWS = 16;
-template <int TW, int VPT, bool EUC = false>
+template <int TW, int VPT, bool EUC = false, bool TM = true>
 __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const StreamCfg& S, SkShared* sh,
                                                   unsigned char* dyn, int64_t r0, int nrow, int v0, int v1,
                                                   const float2* Fold, RingPos& pos, int* abort) {
@@ -582,9 +693,11 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
     int par = 0;
     for (int v = v0; v < v1; ++v)
         for (int j = tid; j < J; j += NC) P.fpart[(int64_t)v * Jp + j] = make_double2(0.0, 0.0);
-    float4 cpi[VPT], crho[VPT];
+    f32x2 cpi[VPT][2], crho[VPT][2];
 #pragma unroll
-    for (int v = 0; v < VPT; ++v) cpi[v] = crho[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int v = 0; v < VPT; ++v) cpi[v][0] = cpi[v][1] = crho[v][0] = crho[v][1] = 0ull;
+    const uint32_t tG = TM ? tmem_G<TW, VPT>(sh->tmem, tm) : 0u;
+    const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
     float errt = 0.f;
     const int nblk = (nrow + rs_ - 1) / rs_;
     const bool want_pi = P.pi != nullptr;
@@ -620,27 +733,42 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
             const int64_t i = r0 + lr;
             const float pf = want_pi ? __ldg(P.p + i) : 0.f;
             float rsum = 0.f;
+            const f32x2 Fh = pack2(F.x, F.x), Fl = pack2(F.y, F.y), ph2 = pack2(phat, phat);
+            __syncwarp();
 #pragma unroll
             for (int v = 0; v < VPT; ++v) {
-                const int col = 4 * (tm.tl + TT * v);
-                if (chunk_inside<TW, VPT>(v) || col < J) {
-                    float4 x = EUC ? euclid_chunk(dxy, rx, rx + Jp, col, J) : *reinterpret_cast<const float4*>(row + col);
-                    float4 gv = *reinterpret_cast<const float4*>(Gs + col);
-                    float4 gl = *reinterpret_cast<const float4*>(Gs + Jp + col);
+                const bool all_in = chunk_inside<TW, VPT>(v);  // lanes past the row: as in sweep_rows
+                const int at = 4 * (tm.tl + TT * v);
+                const int col = all_in || at < J ? at : 0;
+                f32x2 gh[2], gl[2], c[2], t[2];
+                load_G_chunk<TM>(tG, v, Gs, Jp, col, gh, gl);
+                load_C_chunk<EUC>(row, dxy, rx, Jp, J, col, c);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float cost = comp(x, c);
-                        float t = ex2(expo2(F.x, F.y + comp(gl, c), comp(gv, c), cost, P.k_hi, P.k_lo));
-                        if (!chunk_inside<TW, VPT>(v) && col + c >= J) t = 0.f;  // past the row
-                        rsum += t;
-                        comp(cpi[v], c) = fmaf(phat, t, comp(cpi[v], c));
-                        comp(crho[v], c) = fmaf(phat, t > 0.f ? cost * t : 0.f, comp(crho[v], c));
-                        comp(x, c) = t;
+                for (int h = 0; h < 2; ++h) {
+                    const float2 x =
+                        unpack2(add2(add2(fma2(c[h], nk_hi, Fh), gh[h]), fma2(c[h], nk_lo, add2(Fl, gl[h]))));
+                    float2 e = unpack2(c[h]);
+                    float t0 = ex2(x.x), t1 = ex2(x.y);
+                    // a +inf cost (no link, no mass) counts as a finite one; past the row neither does
+                    e.x = fminf(e.x, FLT_MAX);
+                    e.y = fminf(e.y, FLT_MAX);
+                    if (!all_in) {
+                        if (at + 2 * h >= J) t0 = e.x = 0.f;
+                        if (at + 2 * h + 1 >= J) t1 = e.y = 0.f;
                     }
-                    if (want_pi)  // one uniform branch per chunk, not per cell
+                    rsum += t0;
+                    rsum += t1;
+                    t[h] = pack2(t0, t1);
+                    cpi[v][h] = fma2(ph2, t[h], cpi[v][h]);
+                    crho[v][h] = fma2(ph2, mul2(pack2(e.x, e.y), t[h]), crho[v][h]);
+                }
+                if (want_pi) {  // one uniform branch per chunk, not per cell
+                    const float2 ta = unpack2(t[0]), tb = unpack2(t[1]);
+                    const float tv[4] = {ta.x, ta.y, tb.x, tb.y};
 #pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (col + c < J) P.pi[i * P.pi_ld + col + c] = pf * comp(x, c);
+                    for (int q = 0; q < 4; ++q)
+                        if (at + q < J) P.pi[i * P.pi_ld + at + q] = pf * tv[q];
+                    __syncwarp();
                 }
             }
             if (defer) {
@@ -680,15 +808,23 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
             // changed the register allocation of the whole solver loop (1.5% slower at 800
             // columns).
             double2* fp = P.fpart + (int64_t)vp * Jp;
+            float4 sum_pi[VPT], sum_rho[VPT];
+#pragma unroll
+            for (int v = 0; v < VPT; ++v) {
+                const float2 a = unpack2(cpi[v][0]), b = unpack2(cpi[v][1]);
+                const float2 c = unpack2(crho[v][0]), d = unpack2(crho[v][1]);
+                sum_pi[v] = make_float4(a.x, a.y, b.x, b.y);
+                sum_rho[v] = make_float4(c.x, c.y, d.x, d.y);
+            }
             if constexpr (TW > 1) {
-                cta_col_sum<TW, VPT>(comb, cpi, J, Jp, tm, [&](int j, float sum) { atomicAdd(&fp[j].x, (double)sum); });
-                cta_col_sum<TW, VPT>(comb, crho, J, Jp, tm, [&](int j, float sum) { atomicAdd(&fp[j].y, (double)sum); });
+                cta_col_sum<TW, VPT>(comb, sum_pi, J, Jp, tm, [&](int j, float sum) { atomicAdd(&fp[j].x, (double)sum); });
+                cta_col_sum<TW, VPT>(comb, sum_rho, J, Jp, tm, [&](int j, float sum) { atomicAdd(&fp[j].y, (double)sum); });
             } else {
-                cta_col_sum<TW, VPT>(comb, cpi, J, Jp, tm, [&](int j, float sum) { fp[j].x += (double)sum; });
-                cta_col_sum<TW, VPT>(comb, crho, J, Jp, tm, [&](int j, float sum) { fp[j].y += (double)sum; });
+                cta_col_sum<TW, VPT>(comb, sum_pi, J, Jp, tm, [&](int j, float sum) { fp[j].x += (double)sum; });
+                cta_col_sum<TW, VPT>(comb, sum_rho, J, Jp, tm, [&](int j, float sum) { fp[j].y += (double)sum; });
             }
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) cpi[v] = crho[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int v = 0; v < VPT; ++v) cpi[v][0] = cpi[v][1] = crho[v][0] = crho[v][1] = 0ull;
         }
         if (at_end) {
             if (tm.tl == 0) sh->errf[tm.team] = errt;
@@ -711,30 +847,6 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
             const float2 F = Fold[r];
             P.f_nat[r0 + r] = P.eps_ln2 * ((double)F.x + (double)F.y + log2((double)__ldg(P.p + r0 + r)));
         }
-}
-
-// ---- packed FP32 pairs: one instruction for two columns (fma/add .f32x2), each half rounded
-// exactly as the scalar operation rounds it. ------------------------------------------------
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
 }
 
 // Sums of R rows' per-lane values over the team, each in the order of team_reduce; every lane
@@ -783,50 +895,6 @@ __device__ __forceinline__ void team_sum_rows(float (&v)[R], float* red, int nte
     }
 }
 
-// Column potentials in tensor memory: the eight words of chunk v (four high parts, four low
-// parts) of a lane at columns 8 v .. 8 v + 7 of its warp's quarter.  Lane positions repeat
-// every TW warps, so one copy per quarter serves every warp of the CTA (two for teams of 8).
-// The sweep reads G (eight bytes a column) once per row: from shared memory that was two thirds
-// of its shared-memory wavefronts (84 a row of 800 columns, with 25 more for the copy that
-// fills the ring), the busiest unit of the sweep.  Out of tensor memory the sweep of a
-// 50,000 x 800 solve takes 41,000 cycles a CTA instead of 46,600, and the whole solve 0.98 ms
-// instead of 1.00 (1.04 before the packed arithmetic); 100,000 x 1,536: 2.50 ms against 3.03.
-template <int TW, int VPT>
-constexpr int tmem_cols() {
-    constexpr int n = 8 * VPT * (TW == 8 ? 2 : 1);
-    return n <= 32 ? 32 : (n <= 64 ? 64 : 128);
-}
-template <int TW, int VPT>
-__device__ __forceinline__ uint32_t tmem_G(uint32_t base, const Team<TW>& tm) {
-    const uint32_t warp = threadIdx.x >> 5;
-    return base + ((warp & 3u) << 21) + (TW == 8 ? (uint32_t)(tm.wit >> 2) * (8 * VPT) : 0u);
-}
-// Copy G from shared memory to tensor memory (all consumer warps call; G complete in Gs before,
-// visible to every consumer warp after).
-template <int TW, int VPT>
-__device__ __forceinline__ void G_to_tmem(uint32_t base, const float* Gs, int Jp, const Team<TW>& tm) {
-    constexpr int WRITERS = TW == 8 ? 8 : 4, TT = 32 * TW;
-    if ((threadIdx.x >> 5) < WRITERS) {
-        const uint32_t a = tmem_G<TW, VPT>(base, tm);
-        tmem_fence_after();
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            const int col = 4 * (tm.tl + TT * v);
-            float4 hi = make_float4(0.f, 0.f, 0.f, 0.f), lo = hi;
-            if (col < Jp) {
-                hi = *reinterpret_cast<const float4*>(Gs + col);
-                lo = *reinterpret_cast<const float4*>(Gs + Jp + col);
-            }
-            __syncwarp();
-            tmem_st8(a + 8 * v, hi, lo);
-        }
-        tmem_wait_st();
-        tmem_fence_before();
-    }
-    bar_named(CONS_BAR, Cons<TW>::NCW * 32);
-    tmem_fence_after();
-}
-
 // Rows a team takes at once.  Two rows of up to 6 chunks a lane fit the registers (128 a
 // thread); at 7 chunks the second row spills (50,000 x 800: 1.01 ms with two rows, 0.98 with
 // one).  Wider teams stay at one: their rows come from HBM, not L2, at the sizes that matter,
@@ -869,26 +937,12 @@ __device__ __forceinline__ void sweep_rows(const float* (&row)[R], const float2 
         const bool all_in = chunk_inside<TW, VPT>(v);
         const int at = 4 * (tm.tl + TT * v);
         const int col = all_in || at < J ? at : 0;
-        uint32_t w[8];
-        tmem_ld8(tG + 8 * v, w);
         f32x2 gh[2], gl[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            gh[h] = pack2(__uint_as_float(w[2 * h]), __uint_as_float(w[2 * h + 1]));
-            gl[h] = pack2(__uint_as_float(w[4 + 2 * h]), __uint_as_float(w[5 + 2 * h]));
-        }
+        load_G_chunk<true>(tG, v, nullptr, Jp, col, gh, gl);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             f32x2 c[2];
-            if constexpr (EUC) {
-                const float4 e = euclid_chunk(dxy[k], rxs, rxs + Jp, col, J);
-                c[0] = pack2(e.x, e.y);
-                c[1] = pack2(e.z, e.w);
-            } else {
-                const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(row[k] + col);
-                c[0] = e.x;
-                c[1] = e.y;
-            }
+            load_C_chunk<EUC>(row[k], dxy[k], rxs, Jp, J, col, c);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 // the exponent of expo2, two columns at a time
@@ -1121,6 +1175,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         for (int r = tid; r < nrow; r += NC) Fs[r] = P.F_in[r0 + r];
         load_G_smem(P.G_in, J, Jp, Gs, tid, NC);
         bar_named(CONS_BAR, NC);
+        G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
         *ret_par = 0;
         sk_finalize_sweep<TW, VPT, EUC>(P, S, sh, dyn, r0, nrow, v0, v1, Fs, pos, g.abort);
         if (tid == 0) s_stop = 1;
@@ -1128,6 +1183,9 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     }
     load_G_pairs(gs_pairs(P.G, Jp), J, Jp, Gs, tid, NC);
     bar_named(CONS_BAR, NC);
+    G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
+    const uint32_t tG = tmem_G<TW, VPT>(sh->tmem, tm);
+    const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
     int par = 0;
 
     // ---- sweep 1: the log-domain iteration from G^0 with a fixed column scale --------------
@@ -1139,9 +1197,9 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     unsigned long long* flag1 = ACC + Jp + 1;  // zeroed with the totals in setup
     bool exact1 = false;
     {
-        float4 acc[VPT];
+        f32x2 acc[VPT][2];
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
         float2* F1 = Fs + S.rmax;  // F'^1 lives in buffer 1
         int kb = 0;
         for (int vp = v0; vp < v1; ++vp) {
@@ -1156,31 +1214,47 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 for (int j = 0; ok && j < S.rpt; ++j) {
                     const int rr = tm.team + NTEAMS * j;
                     if (rr >= rows) break;
-                    float4 x[VPT];
-                    if constexpr (EUC)
-                        euclid_row<TW, VPT>(__ldg(P.dev_xy + r0 + lr0 + rr), rxs, rxs + Jp, J, tm.tl, x);
-                    else
-                        load_row_smem<TW, VPT>(stage + (size_t)rr * P.ld, J, tm.tl, x);
+                    const float* row = stage + (size_t)rr * P.ld;
+                    const float2 dxy = EUC ? __ldg(P.dev_xy + r0 + lr0 + rr) : make_float2(0.f, 0.f);
+                    f32x2 x[VPT][2];
                     float m = -INFINITY;  // row maximum of G^0 - k C (approximate: only a shift)
+                    __syncwarp();
 #pragma unroll
-                    for (int v = 0; v < VPT; ++v) {
-                        const int col = 4 * (tm.tl + TT * v);
-                        float4 gv = col < Jp ? *reinterpret_cast<const float4*>(Gs + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int v = 0; v < VPT; ++v) {  // lanes past the row: as in sweep_rows
+                        const bool all_in = chunk_inside<TW, VPT>(v);
+                        const int at = 4 * (tm.tl + TT * v);
+                        const int col = all_in || at < J ? at : 0;
+                        f32x2 gh[2], gl[2];
+                        load_G_chunk<true>(tG, v, nullptr, Jp, col, gh, gl);
+                        load_C_chunk<EUC>(row, dxy, rxs, Jp, J, col, x[v]);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) m = fmaxf(m, fmaf(-comp(x[v], c), P.k_hi, comp(gv, c)));
+                        for (int h = 0; h < 2; ++h) {
+                            const float2 y = unpack2(fma2(x[v][h], nk_hi, gh[h]));
+                            if (all_in || at + 2 * h < J) m = fmaxf(m, y.x);
+                            if (all_in || at + 2 * h + 1 < J) m = fmaxf(m, y.y);
+                        }
                     }
                     m = team_reduce<TW, float, true>(m, red, NTEAMS, tm, par);
+                    const f32x2 nm = pack2(-m, -m);
                     float sum = 0.f;
+                    __syncwarp();
 #pragma unroll
                     for (int v = 0; v < VPT; ++v) {
-                        const int col = 4 * (tm.tl + TT * v);
-                        float4 gv = col < Jp ? *reinterpret_cast<const float4*>(Gs + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        float4 gl = col < Jp ? *reinterpret_cast<const float4*>(Gs + Jp + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const bool all_in = chunk_inside<TW, VPT>(v);
+                        const int at = 4 * (tm.tl + TT * v);
+                        f32x2 gh[2], gl[2];
+                        load_G_chunk<true>(tG, v, nullptr, Jp, at, gh, gl);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float t = ex2(expo2(-m, comp(gl, c), comp(gv, c), comp(x[v], c), P.k_hi, P.k_lo));
-                            comp(x[v], c) = t;
-                            sum += t;
+                        for (int h = 0; h < 2; ++h) {
+                            const float2 y = unpack2(add2(add2(fma2(x[v][h], nk_hi, nm), gh[h]), fma2(x[v][h], nk_lo, gl[h])));
+                            float t0 = ex2(y.x), t1 = ex2(y.y);
+                            if (!all_in) {
+                                t0 = at + 2 * h < J ? t0 : 0.f;
+                                t1 = at + 2 * h + 1 < J ? t1 : 0.f;
+                            }
+                            sum += t0;
+                            sum += t1;
+                            x[v][h] = pack2(t0, t1);
                         }
                     }
                     sum = team_reduce<TW, float, false>(sum, red, NTEAMS, tm, par);
@@ -1191,12 +1265,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                         F1[lr0 + rr] = make_float2(-hi, -lo);
                     }
                     const float w = __fdividef(Ps[lr0 + rr], sum) * 0x1p64f;  // p^_i 2^64 / sum
+                    const f32x2 w2 = pack2(w, w);
 #pragma unroll
                     for (int v = 0; v < VPT; ++v) {
-                        acc[v].x = fmaf(x[v].x, w, acc[v].x);
-                        acc[v].y = fmaf(x[v].y, w, acc[v].y);
-                        acc[v].z = fmaf(x[v].z, w, acc[v].z);
-                        acc[v].w = fmaf(x[v].w, w, acc[v].w);
+                        acc[v][0] = fma2(x[v][0], w2, acc[v][0]);
+                        acc[v][1] = fma2(x[v][1], w2, acc[v][1]);
                     }
                 }
                 __syncwarp();
@@ -1204,10 +1277,16 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 pos.next(S.stages);
             }
             float* cp = P.colpart + (int64_t)vp * Jp;
-            cta_col_sum<TW, VPT>(comb, acc, J, Jp, tm, [&](int j, float sum) { cp[j] = sum; });
+            float4 part[VPT];
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int v = 0; v < VPT; ++v) {
+                const float2 u = unpack2(acc[v][0]), w = unpack2(acc[v][1]);
+                part[v] = make_float4(u.x, u.y, w.x, w.y);
+                acc[v][0] = acc[v][1] = 0ull;
+            }
+            cta_col_sum<TW, VPT>(comb, part, J, Jp, tm, [&](int j, float sum) { cp[j] = sum; });
         }
+        tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
         OTA_BARRIER();
         // G^1_j = G^0_j + log2 q^_j - log2(column sum of pi^(1/2)), one warp per column
         {
@@ -1453,9 +1532,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     // a step takes two blocks where a team's rows of one do not fill its passes, if the ring has
     // stages to spare for that
     const int step_blocks = S.rpt % RPP != 0 && S.stages >= 4 ? 2 : 1;
-    const uint32_t tG = tmem_G<TW, VPT>(sh->tmem, tm);
     G_to_tmem<TW, VPT>(sh->tmem, Gs, Jp, tm);
-    const f32x2 nk_hi = pack2(-P.k_hi, -P.k_hi), nk_lo = pack2(-P.k_lo, -P.k_lo);
     for (int s = 2;; ++s) {
         unsigned long long* acc_s = ACC + (size_t)(s & 1) * (Jp + 4);
         const float2* Fold = Fs + ((s - 1) & 1) * S.rmax;  // F'^(s-1)

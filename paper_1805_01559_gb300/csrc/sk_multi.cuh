@@ -629,7 +629,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
         StreamCfg Ss = S;
         Ss.off_G = S.off_G + (int)(sizeof(float) * (size_t)2 * s * Jp);
         const float2* Fold = Fbase + (size_t)s * 2 * S.rmax + retp[s] * S.rmax;
-        sk_finalize_sweep<TW, VPT>(M.P[s], Ss, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
+        sk_finalize_sweep<TW, VPT, false, false>(M.P[s], Ss, sh, dyn, r0, nrow, v0, v1, Fold, pos, g.abort);
         bar_named(CONS_BAR, NC);
     }
     if (tid == 0) s_stop = 1;
