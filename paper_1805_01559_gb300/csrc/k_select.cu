@@ -20,7 +20,7 @@
 // about a million entries the trips between passes.  As eleven launches (four for the sample,
 // four for the candidates, at 7 to 10 us each) the median took 150 us of the 330 us that rates,
 // cost and median of 50,000 x 800 take, and half of the 100 us of a 1000 x 50 cell.
-// Now one launch of 79 us there (18 us on 1000 x 50): 323 -> 277 us and 99 -> 67 us.
+// Now one launch of 70 us there (18 us on 1000 x 50).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -32,17 +32,17 @@
 
 namespace ota {
 
-static constexpr int RS_NT = 1024;               // threads of a CTA (one CTA an SM)
+static constexpr int RS_NT = 512;                // threads of a CTA (one CTA an SM)
 static constexpr int RS_BITS = 11;
 static constexpr int RS_BINS = 1 << RS_BITS;
 static constexpr int RS_PASSES = (32 + RS_BITS - 1) / RS_BITS;
-static constexpr int RS_PER = 8;                 // sample entries a thread
+static constexpr int RS_PER = 16;                // sample entries a thread
 static constexpr int64_t SAMPLE = RS_NT * RS_PER;
 
 // Order-preserving map float bits -> unsigned key (negative values reversed).
 __device__ __forceinline__ uint32_t fkey(float f) {
     const uint32_t u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return u ^ ((uint32_t)((int)u >> 31) | 0x80000000u);
 }
 __device__ __forceinline__ float fkey_inv(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
@@ -99,55 +99,67 @@ __device__ __forceinline__ void load_chunk(const SelSrc& src, int64_t t, int64_t
 
 struct SelShared {
     unsigned h[2][RS_BINS];
-    unsigned long long warp_sum[RS_NT / 32];
-    int digit, ok;
-    long long rank;
+    unsigned long long warp_sum[2][RS_NT / 32];
+    int digit[2], ok;
+    long long rank[2];
     unsigned long long below[RS_NT / 32];
 };
 
-// Digit of the entry of rank `rank` in a histogram of RS_BINS counts (the whole block calls; bin
-// counts by `count`): the digit d with excl(d) <= rank < excl(d) + count(d), and rank - excl(d).
-template <typename Count>
-__device__ __forceinline__ void block_pick(Count count, long long* rank, uint32_t* digit, SelShared* sh) {
-    constexpr int PER = RS_BINS / RS_NT;
+// Digits of two targets in their histograms of RS_BINS counts, count(0, bin) and, where the two
+// differ (NH = 2), count(1, bin), in one block scan: the digit d of target t with excl(d) <=
+// rank[t] < excl(d) + count(d), and rank[t] - excl(d).  The whole block calls.
+template <int NH, typename Count>
+__device__ __forceinline__ void block_pick(Count count, long long (&rank)[2], uint32_t (&digit)[2], SelShared* sh) {
+    constexpr int PER = RS_BINS / RS_NT, NW = RS_NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    unsigned long long c[PER], sum = 0;
+    unsigned long long c[NH][PER], sum[NH], incl[NH];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        c[k] = count(tid * PER + k);
-        sum += c[k];
-    }
-    unsigned long long incl = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
+    for (int h = 0; h < NH; ++h) {
+        sum[h] = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            c[h][k] = count(h, tid * PER + k);
+            sum[h] += c[h][k];
+        }
+        incl[h] = sum[h];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl[h], o);
+            if (lane >= o) incl[h] += y;
+        }
     }
     __syncthreads();  // the shared words may still be read from the last pick
-    if (lane == 31) sh->warp_sum[w] = incl;
-    if (tid == 0) {
-        sh->digit = RS_BINS - 1;  // kept only for an out-of-range rank, which cannot occur
-        sh->rank = *rank;
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+        if (lane == 31) sh->warp_sum[h][w] = incl[h];
+    if (tid < 2) {
+        sh->digit[tid] = RS_BINS - 1;  // kept only for an out-of-range rank, which cannot occur
+        sh->rank[tid] = rank[tid];
     }
     __syncthreads();
-    unsigned long long before = 0;  // the warp totals before this one
-    {
-        const unsigned long long t = lane < w ? sh->warp_sum[lane] : 0ull;
-        before = t;
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+        unsigned long long before = lane < w && lane < NW ? sh->warp_sum[h][lane] : 0ull;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-    }
-    long long excl = (long long)(before + incl - sum);
+        long long excl = (long long)(before + incl[h] - sum[h]);
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        if (c[k] && *rank >= excl && *rank < excl + (long long)c[k]) {
-            sh->digit = tid * PER + k;
-            sh->rank = *rank - excl;
+        for (int k = 0; k < PER; ++k) {
+#pragma unroll
+            for (int t = NH == 1 ? 0 : h; t < (NH == 1 ? 2 : h + 1); ++t)
+                if (c[h][k] && rank[t] >= excl && rank[t] < excl + (long long)c[h][k]) {
+                    sh->digit[t] = tid * PER + k;
+                    sh->rank[t] = rank[t] - excl;
+                }
+            excl += (long long)c[h][k];
         }
-        excl += (long long)c[k];
     }
     __syncthreads();
-    *digit = (uint32_t)sh->digit;
-    *rank = sh->rank;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        digit[t] = (uint32_t)sh->digit[t];
+        rank[t] = sh->rank[t];
+    }
 }
 
 // The two targets of a radix select, the same in every thread.
@@ -167,23 +179,23 @@ struct Targets {
     }
     template <typename Count>
     __device__ __forceinline__ void pick(Count c, SelShared* sh) {
-        const int w = width(), other = same() ? 0 : 1;
-        uint32_t d0, d1;
-        block_pick([&](int b) { return c(0, b); }, &rank[0], &d0, sh);
-        block_pick([&](int b) { return c(other, b); }, &rank[1], &d1, sh);
-        prefix[0] = (prefix[0] << w) | d0;
-        prefix[1] = (prefix[1] << w) | d1;
+        const int w = width();
+        uint32_t d[2];
+        if (same()) block_pick<1>(c, rank, d, sh);
+        else block_pick<2>(c, rank, d, sh);
+        prefix[0] = (prefix[0] << w) | d[0];
+        prefix[1] = (prefix[1] << w) | d[1];
         done += w;
     }
 };
 
-__device__ __forceinline__ void clear_hist(SelShared* sh) {
+__device__ __forceinline__ void clear_hist(SelShared* sh, int nh) {
     __syncthreads();
-    for (int t = threadIdx.x; t < 2 * RS_BINS; t += RS_NT) (&sh->h[0][0])[t] = 0u;
+    for (int t = threadIdx.x; t < nh * RS_BINS; t += RS_NT) (&sh->h[0][0])[t] = 0u;
     __syncthreads();
 }
 
-static constexpr int RS_UNROLL = 4;
+static constexpr int RS_UNROLL = 8;
 static constexpr int RS_GROUP = 32 * RS_UNROLL * 4;  // entries a warp tests per iteration
 static constexpr int RS_STAGE = RS_GROUP + 256;      // entries a warp stages before it writes them out
 static constexpr size_t RS_SMEM = sizeof(SelShared) + sizeof(float) * (RS_NT / 32) * RS_STAGE;
@@ -232,7 +244,7 @@ __global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, lon
             }
         }
         for (int pass = 0; pass < RS_PASSES; ++pass) {
-            clear_hist(sh);
+            clear_hist(sh, B.same() ? 1 : 2);
 #pragma unroll
             for (int e = 0; e < RS_PER; ++e) B.count(sh, v[e]);
             __syncthreads();
@@ -257,7 +269,57 @@ __global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, lon
         };
         const int64_t gwarp = (int64_t)blockIdx.x * (RS_NT / 32) + warp, nwarps = (int64_t)nb * (RS_NT / 32);
         // whole warps walk the chunk space together (the compaction uses warp ballots)
-        for (int64_t t0 = gwarp * 32 * RS_UNROLL; t0 < nch; t0 += nwarps * 32 * RS_UNROLL) {
+        int64_t t0 = gwarp * 32 * RS_UNROLL;
+        if (src.flat && src.vec) {
+            // One aligned run: whole groups without a check per entry.  A lane notes which of its
+            // 32 entries are inside, the warp's lanes find their places by one scan, and only the
+            // noted entries (one or two a lane) are touched again.
+            const int64_t whole = n / RS_GROUP * (RS_GROUP / 4);  // chunks in whole groups
+            const float4* p4 = reinterpret_cast<const float4*>(src.x) + lane;
+            const uint32_t span = kh - kl;
+            const int64_t stride = nwarps * 32 * RS_UNROLL;
+            float4 nx[RS_UNROLL];  // the next group, on the way while this one is tested
+#pragma unroll
+            for (int u = 0; u < RS_UNROLL; ++u)
+                nx[u] = t0 < whole ? __ldg(p4 + t0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (; t0 < whole; t0 += stride) {
+                float x[4 * RS_UNROLL];
+#pragma unroll
+                for (int u = 0; u < RS_UNROLL; ++u) {
+                    x[4 * u] = nx[u].x;
+                    x[4 * u + 1] = nx[u].y;
+                    x[4 * u + 2] = nx[u].z;
+                    x[4 * u + 3] = nx[u].w;
+                }
+                if (t0 + stride < whole)
+#pragma unroll
+                    for (int u = 0; u < RS_UNROLL; ++u) nx[u] = __ldg(p4 + t0 + stride + 32 * u);
+                unsigned lt = 0, in = 0;
+#pragma unroll
+                for (int e = 0; e < 4 * RS_UNROLL; ++e) {
+                    const uint32_t d = fkey(x[e]) - kl;  // below lo wraps around, and past span
+                    if (d <= span) in |= 1u << e;
+                    if (fkey(x[e]) < kl) ++lt;
+                }
+                below += lt;
+                unsigned at = __popc(in);
+                unsigned incl = at;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+                at = fill + incl - at;
+#pragma unroll
+                for (int e = 0; e < 4 * RS_UNROLL; ++e)
+                    if (in >> e & 1u) wb[at++] = x[e];
+                fill += total;
+                if (fill > RS_STAGE - RS_GROUP) flush();  // keep room for one more iteration
+            }
+            // what is left, less than one group, falls to the warp whose turn it is
+        }
+        for (; t0 < nch; t0 += nwarps * 32 * RS_UNROLL) {
             float x[RS_UNROLL][4];
             bool ok[RS_UNROLL][4];
 #pragma unroll
@@ -303,7 +365,8 @@ __global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, lon
     // ---- radix select over the candidates, or over all entries ----------------------------------
     const int64_t m = n_chunks(src);
     for (int pass = 0; T.done < 32; ++pass) {
-        clear_hist(sh);
+        const int nh = T.same() ? 1 : 2;  // histograms in use
+        clear_hist(sh, nh);
         for (int64_t t = (int64_t)blockIdx.x * RS_NT + tid; t < m; t += (int64_t)nb * RS_NT) {
             float x[4];
             bool ok[4];
@@ -322,7 +385,7 @@ __global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, lon
                 if (ok[e]) T.count(sh, x[e]);
         }
         __syncthreads();
-        for (int t = tid; t < 2 * RS_BINS; t += RS_NT) {
+        for (int t = tid; t < nh * RS_BINS; t += RS_NT) {
             const unsigned c = (&sh->h[0][0])[t];
             if (c) atomicAdd(&st->hist[pass][0][0] + t, (unsigned long long)c);
         }

@@ -140,3 +140,26 @@ def test_median_strided_edges(ctx, shape, kind):
         assert eps == oracle.median(C.cpu().numpy().astype(np.float64))
     flat = torch.from_numpy(x.reshape(-1)).cuda()
     assert ctx.median_f32(flat) == oracle.median(x.astype(np.float64))
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (5, 2), (64, 51), (700, 50), (333, 129), (301, 800), (40, 2049), (9, 8190)])
+@pytest.mark.parametrize("scale", [1.0, 1e-18, 1e12])
+def test_rates_edges_and_scales(ctx, shape, scale):
+    """Rates and cost against the oracle at 1e-6 relative (test_gpu_parity.py) for widths around a
+    chunk, a warp and a block, and for gains scaled in and out of the packed divisions' range;
+    the cost equals the two-call form bit for bit."""
+    from paper_1805_01559_gb300 import instances as ins
+    I, J = shape
+    inst = ins.make_instance("t", I, J, 1000.0, I + J, hotspot=False, traffic_sigma=1.0, marginal="uniform")
+    G32 = (inst.G * scale).astype(np.float32)
+    N0 = inst.N0 * scale
+    G, P = torch.from_numpy(G32).cuda(), torch.from_numpy(inst.P.astype(np.float32)).cuda()
+    pad = torch.full((I, (J + 3) // 4 * 4), float("nan"), dtype=torch.float32, device="cuda")
+    pad[:, :J] = G
+    R = ctx.build_rates(pad[:, :J], P, N0, inst.W_hz)
+    R_or = oracle.rates(G32.astype(np.float64), inst.P.astype(np.float32), N0, inst.W_hz)
+    np.testing.assert_allclose(R.cpu().numpy(), R_or, rtol=1e-6)
+    C, _ = ctx.build_cost_from_gains(G, P, N0, inst.W_hz, inst.mu)
+    C2, _ = ctx.build_cost(R.contiguous(), inst.mu)
+    assert torch.equal(C, C2)
+    np.testing.assert_allclose(C.cpu().numpy(), 1.0 / (inst.mu * R_or), rtol=1e-6)
