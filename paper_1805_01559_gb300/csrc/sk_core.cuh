@@ -556,35 +556,6 @@ __device__ __forceinline__ void cta_col_sum(float* comb, const float4 (&acc)[VPT
     bar_named(CONS_BAR, NC);
 }
 
-// ---- packed FP32 pairs: one instruction for two columns (fma/add .f32x2), each half rounded
-// exactly as the scalar operation rounds it. ------------------------------------------------
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // Column potentials in tensor memory: the eight words of chunk v (four high parts, four low
 // parts) of a lane at columns 8 v .. 8 v + 7 of its warp's quarter.  Lane positions repeat
 // every TW warps, so one copy per quarter serves every warp of the CTA (two for teams of 8).
