@@ -205,8 +205,17 @@ __global__ void __launch_bounds__(256) lp_build(const float* __restrict__ C, int
     }
 }
 
+template <typename T>
+struct LpTmem {
+    static constexpr bool value = Chunk<T>::N == 8;
+};
+
 // Consumer warps of the stored-kernel loop.  Returns false when the launch must end early
 // (failed instance or a wait that gave up).
+// 16-bit kernels keep beta in tensor memory (a lane's eight values of chunk v at words 8 v .., a
+// copy per warp quarter, as the FP32 solver keeps G): read from shared memory with every row it
+// was half of the loop's shared-memory traffic, and its 16 KB at 4,096 columns go to the ring.
+// 400,000 x 4,096 in BF16: 11.64 -> 9.11 ms a solve (the loop 7.1 -> about 4.6).
 // RR: a row's values are read twice from the staged stage (once for the row sum, once for the
 // column partials) instead of being kept in registers, so a lane can hold twice the columns'
 // accumulators and rows of 4096 columns keep narrow teams (more rows in flight per CTA).
@@ -217,13 +226,16 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
     constexpr int N = Chunk<T>::N;
     static_assert(NCW <= 24 && NCW / TW <= 16 && 2 * (NCW / TW) * TW <= 64, "SkShared sizes");
     constexpr int TT = 32 * TW, NTEAMS = NCW / TW, NC = NCW * 32;
+    constexpr bool TMB = LpTmem<T>::value;
     uint64_t* full = reinterpret_cast<uint64_t*>(dyn);
     uint64_t* empty = full + MAX_STAGES;
     float* comb = reinterpret_cast<float*>(dyn + SMEM_HDR);   // [Jp] merge row
-    float* Bs = reinterpret_cast<float*>(dyn + S.off_G);      // [Jp] beta
+    float* Bs = reinterpret_cast<float*>(dyn + S.off_G);      // [Jp] beta (not when in tensor memory)
     float* As = reinterpret_cast<float*>(dyn + S.off_F);      // [2][rmax] alpha
     float* Ps = reinterpret_cast<float*>(dyn + S.off_P);      // [rmax] p^
     const T* ring = reinterpret_cast<const T*>(dyn + S.off_ring);
+    const T* zeros = reinterpret_cast<const T*>(sh->zeros);  // what lanes past the row read
+    if (threadIdx.x < 4) sh->zeros[threadIdx.x] = 0u;         // read after the barriers of the setup
     volatile int& s_stop = sh->s_stop;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
     const int nb = g.nb, b = g.b;
@@ -297,11 +309,43 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
         Ps[r] *= inv_sp_f;
         As[((P.it0) & 1) * S.rmax + r] = 1.0f;  // alpha of the plan the launch starts from
     }
-    for (int j = tid; j < Jp; j += NC) Bs[j] = j < J ? 1.0f : 0.0f;
-    bar_named(CONS_BAR, NC);
+    const Team<TW> tm;
+    // beta of every column (1 when src is null; 0 past the row), visible to every consumer warp
+    auto load_beta = [&](const float* src) {
+        if constexpr (TMB) {
+            if (warp < (TW == 8 ? 8 : 4)) {
+                const uint32_t a = tmem_G<TW, VPT>(sh->tmem, tm);
+                tmem_fence_after();
+#pragma unroll
+                for (int v = 0; v < VPT; ++v) {
+                    const int col = N * (tm.tl + TT * v);
+                    float4 x = make_float4(1.f, 1.f, 1.f, 1.f), y = x;
+                    if (src && col < J) {
+                        x = __ldcg(reinterpret_cast<const float4*>(src + col));
+                        y = __ldcg(reinterpret_cast<const float4*>(src + col + 4));
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        comp(x, c) = col + c < J ? comp(x, c) : 0.f;
+                        comp(y, c) = col + 4 + c < J ? comp(y, c) : 0.f;
+                    }
+                    __syncwarp();
+                    tmem_st8(a + 8 * v, x, y);
+                }
+                tmem_wait_st();
+                tmem_fence_before();
+            }
+            bar_named(CONS_BAR, NC);
+            tmem_fence_after();
+        } else {
+            for (int j = tid; j < Jp; j += NC) Bs[j] = j < J ? (src ? src[j] : 1.0f) : 0.f;
+            bar_named(CONS_BAR, NC);
+        }
+    };
+    load_beta(nullptr);
+    const uint32_t tB = TMB ? tmem_G<TW, VPT>(sh->tmem, tm) : 0u;
     LP_BARRIER();  // the sums in errpart are read everywhere before the loop reuses errpart
 
-    const Team<TW> tm;
     uint32_t cseq = 0;
     int par = 0;
     float2* errp = reinterpret_cast<float2*>(P.errpart);
@@ -309,11 +353,11 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
     for (int s = P.it0 + 1;; ++s) {
         const float* Aold = As + ((s - 1) & 1) * S.rmax;
         float* Anew = As + (s & 1) * S.rmax;
-        float acc[VPT][N];
+        f32x2 acc[VPT][N / 2];
 #pragma unroll
         for (int v = 0; v < VPT; ++v)
 #pragma unroll
-            for (int e = 0; e < N; ++e) acc[v][e] = 0.f;
+            for (int e = 0; e < N / 2; ++e) acc[v][e] = 0ull;
         float errt = 0.f;
         int absorb = 0, numeric = 0;
         int kb = 0;
@@ -331,13 +375,20 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
                     if (rr >= rows) break;
                     const int lr = lr0 + rr;
                     const T* row = stage + (size_t)rr * P.ldk;
-                    float x[RR ? 1 : VPT][N];
+                    f32x2 x[RR ? 1 : VPT][N / 2];
                     float ssum = 0.f;
+                    __syncwarp();
 #pragma unroll
                     for (int v = 0; v < VPT; ++v) {
                         const int col = N * (tm.tl + TT * v);
                         float xv[N];
-                        if (col < J) {
+                        if constexpr (TMB) {  // no branch: the warp stays converged
+                            Chunk<T>::load(col < J ? row + col : zeros, xv);
+                            uint32_t w[8];
+                            tmem_ld8(tB + 8 * v, w);
+#pragma unroll
+                            for (int e = 0; e < N; ++e) ssum = fmaf(xv[e], __uint_as_float(w[e]), ssum);
+                        } else if (col < J) {
                             Chunk<T>::load(row + col, xv);
 #pragma unroll
                             for (int e = 0; e < N; e += 4) {  // beta four at a time (16-byte loads)
@@ -353,7 +404,7 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
                         }
                         if constexpr (!RR)
 #pragma unroll
-                            for (int e = 0; e < N; ++e) x[v][e] = xv[e];
+                            for (int e = 0; e < N / 2; ++e) x[v][e] = pack2(xv[2 * e], xv[2 * e + 1]);
                     }
                     ssum = team_reduce<TW, float, false>(ssum, sh->red, NTEAMS, tm, par);
                     const float ph = Ps[lr];
@@ -363,22 +414,22 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
                     absorb |= fabsf(__log2f(an)) > tau;
                     if (tm.tl == 0) Anew[lr] = an;
                     const float w = ph * an;
+                    const f32x2 w2 = pack2(w, w);
                     if constexpr (RR) {
 #pragma unroll
                         for (int v = 0; v < VPT; ++v) {
                             const int col = N * (tm.tl + TT * v);
-                            if (col < J) {
-                                float xv[N];
-                                Chunk<T>::load(row + col, xv);
+                            float xv[N];
+                            Chunk<T>::load(col < J ? row + col : zeros, xv);
 #pragma unroll
-                                for (int e = 0; e < N; ++e) acc[v][e] = fmaf(xv[e], w, acc[v][e]);
-                            }
+                            for (int e = 0; e < N / 2; ++e)
+                                acc[v][e] = fma2(pack2(xv[2 * e], xv[2 * e + 1]), w2, acc[v][e]);
                         }
                     } else {
 #pragma unroll
                         for (int v = 0; v < VPT; ++v)
 #pragma unroll
-                            for (int e = 0; e < N; ++e) acc[v][e] = fmaf(x[v][e], w, acc[v][e]);
+                            for (int e = 0; e < N / 2; ++e) acc[v][e] = fma2(x[v][e], w2, acc[v][e]);
                     }
                 }
                 __syncwarp();
@@ -399,10 +450,11 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
                             for (int e = 0; e < N; e += 4) {
                                 float4* d = reinterpret_cast<float4*>(comb + col + e);
                                 float4 o = t == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : *d;
-                                o.x += acc[v][e];
-                                o.y += acc[v][e + 1];
-                                o.z += acc[v][e + 2];
-                                o.w += acc[v][e + 3];
+                                const float2 lo = unpack2(acc[v][e / 2]), hi = unpack2(acc[v][e / 2 + 1]);
+                                o.x += lo.x;
+                                o.y += lo.y;
+                                o.z += hi.x;
+                                o.w += hi.y;
                                 *d = o;
                             }
                     }
@@ -419,10 +471,11 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
 #pragma unroll
             for (int v = 0; v < VPT; ++v)
 #pragma unroll
-                for (int e = 0; e < N; ++e) acc[v][e] = 0.f;
+                for (int e = 0; e < N / 2; ++e) acc[v][e] = 0ull;
             errt = 0.f;
             bar_named(CONS_BAR, NC);  // comb and errf are free again
         }
+        if (TMB) tmem_fence_before();  // this sweep's reads of beta, before the barriers that precede its next copy
         if (__any_sync(0xffffffffu, numeric) && lane == 0) atomicCAS(status, DEV_OK, DEV_ENUMERIC);
         if (__any_sync(0xffffffffu, absorb) && lane == 0) atomicOr(&P.st->absorb[s & 1], 1);
         LP_BARRIER();
@@ -493,8 +546,7 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
             if (tid == 0) s_stop = 1;
             return true;
         }
-        for (int j = tid; j < Jp; j += NC) Bs[j] = j < J ? Bnew[j] : 0.f;
-        bar_named(CONS_BAR, NC);
+        load_beta(Bnew);
     }
 #undef LP_BARRIER
 }
@@ -518,6 +570,7 @@ __global__ void __launch_bounds__(32 * (NCW + 1), 1) lp_loop(LpParams P, StreamC
         sh.s_bad = 0;
         mbar_fence_init();
     }
+    if (LpTmem<T>::value && warp == 0) tmem_alloc(&sh.tmem, tmem_cols<TW, VPT>());
     __syncthreads();
     if (warp == NCW) {
         if (lane == 0)
@@ -527,6 +580,10 @@ __global__ void __launch_bounds__(32 * (NCW + 1), 1) lp_loop(LpParams P, StreamC
     }
     GroupCtx g{(int)gridDim.x, (int)blockIdx.x, &P.st->bar, 0u, &P.st->status, &P.st->status};
     lp_consumers<T, TW, VPT, RR, NCW>(P, S, g, &sh, dyn, r0, r1);
+    if (LpTmem<T>::value) {
+        bar_named(CONS_BAR, NCW * 32);
+        if (warp == 0) tmem_free(sh.tmem, tmem_cols<TW, VPT>());
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -596,6 +653,10 @@ ot_status lowp_solve_t(ot_assoc_ctx* ctx, const SolveArgs& a, double absorb_log2
     if (!plan_stage(nteams, I, Jp, ldk, grid, 24576, 232448 - 4096, &S, &smem, &V, (int)sizeof(T), 1, 4, 1))
         return set_error(ctx, OT_EUNSUPPORTED, "stored kernel does not fit the shared memory (I=%lld J=%d)",
                          (long long)I, J);
+    // beta in tensor memory: its room goes to the ring (the instances accepted stay the same)
+    if (LpTmem<T>::value &&
+        !plan_stage(nteams, I, Jp, ldk, grid, 24576, 232448 - 4096, &S, &smem, &V, (int)sizeof(T), 0, 4, 1))
+        return set_error(ctx, OT_EUNSUPPORTED, "stored-kernel geometry");
     if (allow_max_dynamic_smem(kk.fn, smem) != cudaSuccess) {
         cudaGetLastError();
         return set_error(ctx, OT_ECUDA, "stored-kernel loop: shared memory");

@@ -22,9 +22,9 @@
 // Each CTA owns a fixed block-aligned range of rows for the whole solve; its row potentials
 // (an FP32 hi/lo pair, updated with error-free FP32 two-sums) and p^ live in shared memory.
 // A producer warp streams the CTA's rows of C through a ring of shared-memory stages with
-// bulk copies (TMA); it runs on into the next sweep while the consumers are in a grid
-// barrier (C never changes).  Column partials are combined per CTA in team order and
-// across CTAs in CTA order, so reruns are bit-identical.  Every wait is bounded.
+// bulk copies (TMA); it runs on into the next sweep while the consumers wait for the column
+// totals (C never changes).  Column partials are combined per CTA in team order and across
+// partitions as integers, so reruns are bit-identical.  Every wait is bounded.
 #include <cuda_runtime.h>
 #include <math.h>
 

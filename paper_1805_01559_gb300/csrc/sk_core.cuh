@@ -464,6 +464,7 @@ __device__ __forceinline__ void warp_sum_pair(float& s, float& e) {
 
 // Shared-memory words of the consumer warps (and the producer's stop flag).
 struct SkShared {
+    alignas(16) unsigned zeros[4];  // a chunk of zeros (stored-kernel loop)
     float red[64];          // team reductions: 2 * NTEAMS * TW <= 24 values (float2 pairs: 48 floats)
     float errf[16];         // per-team row residuals
     double sh_sum[24][2];   // per-warp setup sums (up to 24 consumer warps)
