@@ -323,8 +323,6 @@ ot_status ot_assoc_build_cost_from_gains(ot_assoc_ctx* ctx, const float* G, int6
     if (st) return st;
     unsigned long long* bad = &state->bad;
     double* med = state->med;
-    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_error(ctx, e, "memset");
     st = launch_rates(ctx, G, ld_g, P, I, (int)J, N0, W_hz, R_out, ld_r, s, mu, C_out, ld_c, bad);
     if (st) return st;
     if (!eps_out) return OT_OK;
@@ -332,7 +330,7 @@ ot_status ot_assoc_build_cost_from_gains(ot_assoc_ctx* ctx, const float* G, int6
     if (st) return st;
     CostState* h = (CostState*)host_staging(ctx, sizeof(CostState), &st);
     if (st) return st;
-    e = cudaMemcpyAsync(h, state, sizeof(CostState), cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(h, state, sizeof(CostState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "build_cost_from_gains");
     if (h->bad) return set_error(ctx, OT_EINVAL, "%llu rate entries are not finite and > 0", h->bad);

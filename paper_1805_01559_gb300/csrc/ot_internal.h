@@ -151,7 +151,7 @@ ot_status f32_finalize_on(ot_assoc_ctx* ctx, const SolveArgs& a, const float2* F
                           double err, int converged, SolveSummary* sum_host);
 
 // Rates into R (may be null when C is given); with C non-null also C = (1/mu)/R in the same
-// pass, counting rates that are not finite and > 0 into *bad_dev.
+// pass, counting rates that are not finite and > 0 into *bad_dev (which it clears first).
 ot_status launch_rates(ot_assoc_ctx* ctx, const float* G, int64_t ld_g, const float* P, int64_t I,
                        int J, double N0, double W, float* R, int64_t ld_r, cudaStream_t s, double mu = 1.0,
                        float* C = nullptr, int64_t ld_c = 0, unsigned long long* bad_dev = nullptr);
