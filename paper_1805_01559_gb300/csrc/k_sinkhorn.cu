@@ -56,58 +56,68 @@ __global__ void sk_multi_status(const LoopState* grp, LoopState* a, LoopState* b
 // column partials (sum p^ t, sum p^ C t) and row residuals; these kernels finish the column
 // marginals, loads rho_j, potentials g in natural units, and the totals.
 // ------------------------------------------------------------------------------------------
-__global__ void sk_finalize_cols(const double2* __restrict__ fpart, int nb, int Jp, int J,
-                                 const float* __restrict__ q, const DevScalars* sc,
-                                 const LoopState* st, const double* G, int g_by_parity, double eps_ln2,
-                                 double* g_out, double* rrh_load, double2* cols) {
-    if (st->status != DEV_OK) return;
-    if (g_by_parity) G += (st->iters & 1) * Jp;  // G^k of the returned plan
+// The last block to finish its columns forms the totals: row residual (per-partition partials),
+// column residual and transport cost = sum_j rho_j, in a fixed order whichever block it is.  (As a
+// launch of its own it cost small solves about 3 us.)
+__global__ void __launch_bounds__(512) sk_finalize_cols(const double2* __restrict__ fpart, int nb, int Jp, int J,
+                                                        const float* __restrict__ q, const DevScalars* sc,
+                                                        const LoopState* st, const double* G, int g_by_parity,
+                                                        double eps_ln2, double* g_out, double* rrh_load, double2* cols,
+                                                        const double* __restrict__ epart, unsigned* done,
+                                                        SolveSummary* out) {
+    __shared__ double sh[3][8];
+    __shared__ int s_last;
+    const bool ok = st->status == DEV_OK;
     const int lane = threadIdx.x & 31;
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int j = w; j < J; j += nw) {
-        double s = 0.0, r = 0.0;
-        for (int bb = lane; bb < nb; bb += 32) {
-            const double2 v = fpart[(int64_t)bb * Jp + j];
-            s += v.x;
-            r += v.y;
-        }
-        s = warp_sum(s);
-        r = warp_sum(r);
-        if (lane == 0) {
-            cols[j] = make_double2(fabs(s - (double)q[j] * sc->inv_sq), r);
-            if (rrh_load) rrh_load[j] = r * sc->sp;
-            g_out[j] = eps_ln2 * G[j];
+    if (ok) {
+        if (g_by_parity) G += (st->iters & 1) * Jp;  // G^k of the returned plan
+        const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+        const int nw = (gridDim.x * blockDim.x) >> 5;
+        for (int j = w; j < J; j += nw) {
+            double s = 0.0, r = 0.0;
+            for (int bb = lane; bb < nb; bb += 32) {
+                const double2 v = fpart[(int64_t)bb * Jp + j];
+                s += v.x;
+                r += v.y;
+            }
+            s = warp_sum(s);
+            r = warp_sum(r);
+            if (lane == 0) {
+                cols[j] = make_double2(fabs(s - (double)q[j] * sc->inv_sq), r);
+                if (rrh_load) rrh_load[j] = r * sc->sp;
+                g_out[j] = eps_ln2 * G[j];
+            }
         }
     }
-}
-
-// Totals: row residual (per-CTA partials), column residual and transport cost = sum_j rho_j.
-__global__ void sk_summary(const double* __restrict__ epart, int nb, const double2* __restrict__ cols, int J,
-                           const DevScalars* sc, const LoopState* st, SolveSummary* out) {
-    __shared__ double sh[3][32];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     double er = 0.0, co = 0.0, ec = 0.0;
-    const bool ok = st->status == DEV_OK;
-    if (ok) {
-        for (int bb = threadIdx.x; bb < nb; bb += blockDim.x) er += epart[bb];
-        for (int j = threadIdx.x; j < J; j += blockDim.x) {
-            const double2 c = cols[j];
+    if (ok && threadIdx.x < 256) {
+        for (int bb = threadIdx.x; bb < nb; bb += 256) er += epart[bb];
+        for (int j = threadIdx.x; j < J; j += 256) {
+            const double2 c = __ldcg(cols + j);
             ec += c.x;
             co += c.y;
         }
     }
-    er = warp_sum(er);
-    co = warp_sum(co);
-    ec = warp_sum(ec);
-    if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = er;
-        sh[1][threadIdx.x >> 5] = co;
-        sh[2][threadIdx.x >> 5] = ec;
+    if (threadIdx.x < 256) {
+        er = warp_sum(er);
+        co = warp_sum(co);
+        ec = warp_sum(ec);
+        if (lane == 0) {
+            sh[0][threadIdx.x >> 5] = er;
+            sh[1][threadIdx.x >> 5] = co;
+            sh[2][threadIdx.x >> 5] = ec;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, c = 0.0, e = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        for (int w = 0; w < 8; ++w) {
             a += sh[0][w];
             c += sh[1][w];
             e += sh[2][w];
@@ -207,6 +217,9 @@ ot_status plan_solve_uncached(const Kernels& kk, int64_t I, int Jp, int64_t ld, 
     return OT_OK;
 }
 
+// Block counter of the finalize launch: behind the summary, in the state words every solve clears.
+inline unsigned* finalize_counter(SolveSummary* summ) { return (unsigned*)((char*)summ + 256); }
+
 // Device buffers of one solve.
 struct SolveBufs {
     DevScalars* sc;
@@ -299,8 +312,8 @@ cudaError_t enqueue_solve(const SolveArgs& a, const Kernels& kk, const LoopLaunc
         const int nb_cols = (int)std::max<int64_t>(1, std::min<int64_t>((J + 15) / 16, 1024));
         const double* G = mode.G_in ? mode.G_in : B.G;
         sk_finalize_cols<<<nb_cols, 512, 0, s>>>(B.fpart, LL.V, Jp, J, a.q, B.sc, B.ls, G, mode.G_in ? 0 : 1,
-                                                 a.eps * LN2, a.out->g, a.out->rrh_load, B.cols);
-        sk_summary<<<1, 256, 0, s>>>(P.epart, LL.V, B.cols, J, B.sc, B.ls, B.summ);
+                                                 a.eps * LN2, a.out->g, a.out->rrh_load, B.cols, P.epart,
+                                                 finalize_counter(B.summ), B.summ);
     }
     if (ctx) timing_mark(ctx, 3, s);
     return cudaGetLastError();
@@ -347,7 +360,7 @@ ot_status enqueue_solve_f32(ot_assoc_ctx* ctx, const SolveArgs& a, SolveSummary*
     cudaStream_t s = a.stream;
     cudaError_t e = enqueue_solve(a, kk, LL, B, ctx->spin_limit, s, kev0 ? nullptr : ctx, SolveMode(), kev0, kev1);
     if (e != cudaSuccess) return cuda_error(ctx, e, "solve launch");
-    ctx->launches += 3;
+    ctx->launches += 2;
     e = cudaMemcpyAsync(dest, B.summ, sizeof(SolveSummary), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "summary copy");
     return OT_OK;
@@ -482,11 +495,11 @@ ot_status launch_solve_multi(ot_assoc_ctx* ctx, const SolveArgs& a, int n, const
     const int nb_cols = (int)std::max<int64_t>(1, std::min<int64_t>((J + 15) / 16, 1024));
     for (int k = 0; k < n; ++k) {
         sk_finalize_cols<<<nb_cols, 512, 0, s>>>(B[k].fpart, V, Jp, J, a.q, B[k].sc, B[k].ls, B[k].G, 1,
-                                                 eps[k] * LN2, outs[k]->g, outs[k]->rrh_load, B[k].cols);
-        sk_summary<<<1, 256, 0, s>>>(B[k].errpart + V, V, B[k].cols, J, B[k].sc, B[k].ls, B[k].summ);
+                                                 eps[k] * LN2, outs[k]->g, outs[k]->rrh_load, B[k].cols,
+                                                 B[k].errpart + V, finalize_counter(B[k].summ), B[k].summ);
     }
     timing_mark(ctx, 3, s);
-    ctx->launches += 2 + 2 * n;
+    ctx->launches += 2 + n;
     e = cudaGetLastError();
     for (int k = 0; k < n && e == cudaSuccess; ++k)
         e = cudaMemcpyAsync(hsum + k, B[k].summ, sizeof(SolveSummary), cudaMemcpyDeviceToHost, s);
@@ -562,7 +575,7 @@ ot_status f32_finalize_on(ot_assoc_ctx* ctx, const SolveArgs& a, const float2* F
     if (e == cudaSuccess) e = cudaMemcpyAsync(hsum, B.summ, sizeof(SolveSummary), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "finalize");
-    ctx->launches += 4;
+    ctx->launches += 3;
     *sum_host = *hsum;
     return OT_OK;
 }
