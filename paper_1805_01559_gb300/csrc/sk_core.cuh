@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "ot_common.cuh"
+#include "sk_totals.h"
 
 namespace ota {
 
@@ -51,16 +52,7 @@ struct LoopState {
 // The totals are sums of integers, the same in any order, so every CTA reads the same column
 // sums whatever the number of CTAs or the order in which partitions arrive.
 //
-// The words carry their own completion: each partition adds its value plus 1 << 56, and a
-// reader, which knows what the word held when the row was last complete, has the sweep's total
-// once the difference counts all V partitions (V <= 152, a sweep's values stay below 2^56).  So
-// no barrier stands between the sweep and the column update, and nothing is cleared.  A row is
-// added to again two sweeps later, by a CTA that has seen the other row complete, to which
-// every CTA has added after it read this one.
-static constexpr int FX_BITS = 40;   // a column total of q^_j is about 2^40 units
-static constexpr int FX_TOP = 48;    // partials (and totals) from 2^48 on go to the exact path
-static constexpr int FX_ERR = 50;    // row residuals in units of 2^-50
-static constexpr int FX_COUNT = 56;  // bit position of the partition count
+// How the words are counted and when a row may be added to again: sk_totals.h.
 __host__ __device__ constexpr size_t gstate_words(int Jp) { return (size_t)Jp * 15 / 2 + 8; }
 __host__ __device__ constexpr size_t gstate_bytes(int Jp) { return 8 * gstate_words(Jp); }
 __device__ __forceinline__ float2* gs_lq2(double* G, int Jp) { return reinterpret_cast<float2*>(G + 3 * (size_t)Jp); }
@@ -368,10 +360,6 @@ __host__ __device__ __forceinline__ int64_t part_row(int64_t I, int rs, int V, i
     const int64_t B = (I + rs - 1) / rs;
     const int64_t r = (B * v / V) * rs;
     return r < I ? r : I;
-}
-__host__ __device__ __forceinline__ void cta_parts(int V, int b, int nb, int* v0, int* v1) {
-    *v0 = (int)((int64_t)V * b / nb);
-    *v1 = (int)((int64_t)V * (b + 1) / nb);
 }
 // Rows [r0, r1) of CTA b of nb.
 __host__ __device__ __forceinline__ void cta_rows(int64_t I, int rs, int V, int b, int nb, int64_t* r0,
@@ -1591,7 +1579,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
 #pragma unroll
                 for (int t = 0; t < NTEAMS; ++t) e += sh->werr[t];
                 // at most 2^51 in all for a plan of unit mass; a broken plan's must not reach the count
-                atomicAdd(acc_s + Jp, (1ull << FX_COUNT) + (e < (1ull << 52) ? e : 1ull << FX_TOP));
+                atomicAdd(acc_s + Jp, FX_ONE + (e < (1ull << 52) ? e : 1ull << FX_TOP));
             }
             if (tm.team >= HALF) {
 #pragma unroll
@@ -1612,7 +1600,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 cp[j] = sum;
                 const float x = sum * __int_as_float((sxj + 127) << 23);  // S_j <= 126; 0 for "never"
                 const bool fits = sxj != 0 && x < (float)(1ull << FX_TOP);
-                atomicAdd(acc_s + j, (1ull << FX_COUNT) + (fits ? __float2ull_rn(x) : 1ull << FX_TOP));
+                atomicAdd(acc_s + j, FX_ONE + (fits ? __float2ull_rn(x) : 1ull << FX_TOP));
             };
 #pragma unroll
             for (int u = 0; u < CU; ++u)
@@ -1622,6 +1610,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
             if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // comb and werr are free again
         }
+        // a CTA without a partition counts itself into the residual word: it has read the other row
+        if (v0 == v1 && tid == 0) atomicAdd(acc_s + Jp, (unsigned long long)FX_ONE);
         tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
         // G^s_j = G^(s-1)_j + log2 q^_j - log2 s_j, every column in every CTA (FP32 pairs).  The
         // sum s_j is the fixed-point total T_j 2^-S_j; a column whose total is too large or too
@@ -1629,7 +1619,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         unsigned exact = 0;  // of this thread's columns
         int* flags = &sh->flags[s & 1];
         for (int u0 = 0; u0 < UC; u0 += CU) {
-            unsigned long long T[CU], was[CU];
+            unsigned long long A[CU], was[CU];
             float2 lq[CU];
             int sx[CU];
 #pragma unroll
@@ -1639,30 +1629,25 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 lq[u] = in ? __ldcg(LQ2 + j) : make_float2(0.f, 0.f);
                 sx[u] = in ? __ldcg(SX + j) : 0;
                 was[u] = in ? prev[s & 1][u0 + u] : 0ull;
-                T[u] = 0ull;
             }
             const bool first = u0 == 0;
             long long n = 0;
-            for (;;) {  // until every partition's addition to this thread's words has arrived
+            for (;;) {  // until every addition due to this thread's words has arrived
                 bool all = true;
-                unsigned long long A[CU], Ae = 0ull;
+                unsigned long long Ae = 0ull;
 #pragma unroll
                 for (int u = 0; u < CU; ++u) {
                     const int j = tid + (u0 + u) * NC;
-                    A[u] = u0 + u < UC && j < J ? ld_relaxed_u64(acc_s + j) : was[u] + ((unsigned long long)V << FX_COUNT);
+                    A[u] = u0 + u < UC && j < J ? ld_relaxed_u64(acc_s + j) : was[u] + ((unsigned long long)fx_due_col(V) << FX_COUNT);
                 }
                 if (first && tid == 0) Ae = ld_relaxed_u64(acc_s + Jp);
 #pragma unroll
-                for (int u = 0; u < CU; ++u) {
-                    T[u] = A[u] - was[u];
-                    all = all && (T[u] >> FX_COUNT) == (unsigned long long)V;
-                }
+                for (int u = 0; u < CU; ++u) all = all && fx_complete(A[u], was[u], fx_due_col(V));
                 if (first && tid == 0) {
-                    const unsigned long long D = Ae - prev_err[s & 1];
-                    all = all && (D >> FX_COUNT) == (unsigned long long)V;
+                    all = all && fx_complete(Ae, prev_err[s & 1], fx_due_err(V, nb));
                     if (all) {
+                        sh->s_err = fx_value(Ae, prev_err[s & 1]);
                         prev_err[s & 1] = Ae;
-                        sh->s_err = D & ((1ull << FX_COUNT) - 1);
                     }
                 }
                 if (all) {
@@ -1713,11 +1698,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
 #pragma unroll
             for (int u = 0; u < CU; ++u) {
                 const int j = tid + (u0 + u) * NC;
-                T[u] &= (1ull << FX_COUNT) - 1;
+                const unsigned long long T = fx_value(A[u], was[u]);
                 const bool in = u0 + u < UC && j < J;
-                const bool ok = T[u] >= (1ull << 30) && T[u] < (1ull << FX_TOP);
-                const float th = __ull2float_rn(T[u]);
-                const float tl = (float)((long long)T[u] - (long long)__float2ull_rn(th));
+                const bool ok = T >= (1ull << 30) && T < (1ull << FX_TOP);
+                const float th = __ull2float_rn(T);
+                const float tl = (float)((long long)T - (long long)__float2ull_rn(th));
                 float2 ls = df_log2(make_float2(ok ? th : 1.f, ok ? tl : 0.f));
                 ls.x -= (float)sx[u];
                 const float2 d = df_add2(lq[u], make_float2(-ls.x, -ls.y));
