@@ -346,7 +346,7 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
     const uint32_t tB = TMB ? tmem_G<TW, VPT>(sh->tmem, tm) : 0u;
     LP_BARRIER();  // the sums in errpart are read everywhere before the loop reuses errpart
 
-    uint32_t cseq = 0;
+    RingPos pos;
     int par = 0;
     float2* errp = reinterpret_cast<float2*>(P.errpart);
     const float tau = P.tau;
@@ -364,13 +364,12 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
         for (int vp = v0; vp < v1; ++vp) {
             const int vend = pend[vp];
             for (; kb < vend; ++kb) {
-                const int st = (int)(cseq % (uint32_t)S.stages);
-                const uint32_t ph = (cseq / (uint32_t)S.stages) & 1u;
-                const bool ok = mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
+                const int st = pos.st;
+                pos.wait(full, P.spin, g.abort);
                 const int lr0 = kb * rs_;
                 const int rows = min(rs_, nrow - lr0);
                 const T* stage = ring + (size_t)st * S.stage_floats;
-                for (int jr = 0; ok && jr < S.rpt; ++jr) {
+                for (int jr = 0; jr < S.rpt; ++jr) {
                     const int rr = tm.team + NTEAMS * jr;
                     if (rr >= rows) break;
                     const int lr = lr0 + rr;
@@ -433,8 +432,8 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
                     }
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[st]);
-                ++cseq;
+                if (lane == 0) pos.release(empty, st);
+                pos.next(S.stages);
             }
             // end of partition vp: column partials and row residual.  The teams add their
             // partials into one merge row one team after the other (team order), so the

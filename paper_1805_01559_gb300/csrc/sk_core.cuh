@@ -425,10 +425,21 @@ inline bool plan_stage(int nteams, int64_t I, int Jp, int64_t ld, int nb, int st
     return true;
 }
 
-// A consumer's place in the ring of stages: the stage and the parity of its current use.
+// A consumer's place in the ring of stages: the stage and the parity of its current use.  Once a
+// wait for a stage has given up (the launch is ending, and its status says so; bit 1 of ph) a
+// lane neither waits for stages nor releases them any more, but it goes through its rows like the
+// others, on whatever the ring holds: if it left them out, its warp would be torn at the shuffles
+// and its team left waiting at the team's barriers, which have no limit.
 struct RingPos {
     int st = 0;
     uint32_t ph = 0;
+    __device__ __forceinline__ void wait(uint64_t* full, long long spin, int* status) {
+        if (ph < 2u && !mbar_try_wait(&full[st], ph) && !mbar_wait_bounded(&full[st], ph, spin, status)) ph |= 2u;
+    }
+    // by lane 0 of each warp, after the warp's last read of the stage
+    __device__ __forceinline__ void release(uint64_t* empty, int stage) const {
+        if (ph < 2u) mbar_arrive(&empty[stage]);
+    }
     __device__ __forceinline__ void next(int stages) {
         if (++st == stages) {
             st = 0;
@@ -677,12 +688,11 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
     int vend = v0 < v1 ? pend[v0] : 0;
     for (int kb = 0; kb < nblk; ++kb) {
         const int st = pos.st;
-        const uint32_t ph = pos.ph;
-        const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, abort);
+        if (!EUC) pos.wait(full, P.spin, abort);
         const int lr0 = kb * rs_;
         const int rows = min(rs_, nrow - lr0);
         const float* stage = ring + (size_t)st * S.stage_floats;
-        for (int jr = 0; ok && jr < S.rpt; ++jr) {
+        for (int jr = 0; jr < S.rpt; ++jr) {
             const int rr = tm.team + NTEAMS * jr;
             if (rr >= rows) break;
             const int lr = lr0 + rr;
@@ -743,7 +753,7 @@ __device__ __forceinline__ void sk_finalize_sweep(const SolveParams& P, const St
             }
         }
         __syncwarp();
-        if (!EUC && lane == 0) mbar_arrive(&empty[st]);
+        if (!EUC && lane == 0) pos.release(empty, st);
         pos.next(S.stages);
         const bool at_end = (kb + 1 == vend);
         if ((kb + 1 - vbeg) % every == 0 || at_end) {
@@ -1166,12 +1176,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             const int vend = pend[vp];
             for (; kb < vend; ++kb) {
                 const int st = pos.st;
-                const uint32_t ph = pos.ph;
-                const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
+                if (!EUC) pos.wait(full, P.spin, g.abort);
                 const int lr0 = kb * rs_;
                 const int rows = min(rs_, nrow - lr0);
                 const float* stage = ring + (size_t)st * S.stage_floats;
-                for (int j = 0; ok && j < S.rpt; ++j) {
+                for (int j = 0; j < S.rpt; ++j) {
                     const int rr = tm.team + NTEAMS * j;
                     if (rr >= rows) break;
                     const float* row = stage + (size_t)rr * P.ld;
@@ -1233,7 +1242,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                     }
                 }
                 __syncwarp();
-                if (!EUC && lane == 0) mbar_arrive(&empty[st]);
+                if (!EUC && lane == 0) pos.release(empty, st);
                 pos.next(S.stages);
             }
             float* cp = P.colpart + (int64_t)vp * Jp;
@@ -1288,12 +1297,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
           const int vend = pend[vp];
           for (; kb < vend; ++kb) {
             const int st = pos.st;
-            const uint32_t ph = pos.ph;
-            const bool ok = EUC || mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
+            if (!EUC) pos.wait(full, P.spin, g.abort);
             const int lr0 = kb * rs_;
             const int rows = min(rs_, nrow - lr0);
             const float* stage = ring + (size_t)st * S.stage_floats;
-            for (int j = 0; ok && j < S.rpt; ++j) {
+            for (int j = 0; j < S.rpt; ++j) {
                 const int rr = tm.team + NTEAMS * j;
                 if (rr >= rows) break;
                 float4 x[VPT];
@@ -1349,7 +1357,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                     }
             }
             __syncwarp();
-            if (!EUC && lane == 0) mbar_arrive(&empty[st]);
+            if (!EUC && lane == 0) pos.release(empty, st);
             pos.next(S.stages);
           }
             // end of partition vp: merge the teams' (max, sum) pairs in two rounds through
@@ -1507,19 +1515,18 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
           while (kb < vend) {
             // a step: one stage block, or two when a team's rows in a block do not pair up
             const int nblk = min(step_blocks, vend - kb);
-            const RingPos p0 = pos;
-            bool ok = EUC || mbar_try_wait(&full[p0.st], p0.ph) || mbar_wait_bounded(&full[p0.st], p0.ph, P.spin, g.abort);
+            if (!EUC) pos.wait(full, P.spin, g.abort);
+            const int st0 = pos.st;
             pos.next(S.stages);
-            RingPos p1 = pos;
+            const int st1 = pos.st;
             if (nblk == 2) {
-                ok = ok && (EUC || mbar_try_wait(&full[p1.st], p1.ph) ||
-                            mbar_wait_bounded(&full[p1.st], p1.ph, P.spin, g.abort));
+                if (!EUC) pos.wait(full, P.spin, g.abort);
                 pos.next(S.stages);
             }
-            const float* stage0 = ring + (size_t)p0.st * S.stage_floats + (size_t)tm.team * P.ld;
-            const float* stage1 = ring + (size_t)p1.st * S.stage_floats + (size_t)tm.team * P.ld;
+            const float* stage0 = ring + (size_t)st0 * S.stage_floats + (size_t)tm.team * P.ld;
+            const float* stage1 = ring + (size_t)st1 * S.stage_floats + (size_t)tm.team * P.ld;
             const int lr0 = kb * rs_ + tm.team;  // the team's rows are lr0 + NTEAMS q
-            const int nq = ok ? min(nblk * S.rpt, (nrow - lr0 + NTEAMS - 1) / NTEAMS) : 0;
+            const int nq = min(nblk * S.rpt, (nrow - lr0 + NTEAMS - 1) / NTEAMS);
             auto staged = [&](int q) {
                 return q < S.rpt ? stage0 + (size_t)(NTEAMS * q) * P.ld : stage1 + (size_t)(NTEAMS * (q - S.rpt)) * P.ld;
             };
@@ -1549,8 +1556,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             }
             __syncwarp();
             if (!EUC && lane == 0) {
-                mbar_arrive(&empty[p0.st]);
-                if (nblk == 2) mbar_arrive(&empty[p1.st]);
+                pos.release(empty, st0);
+                if (nblk == 2) pos.release(empty, st1);
             }
             kb += nblk;
           }

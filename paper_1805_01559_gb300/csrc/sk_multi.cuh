@@ -102,12 +102,11 @@ __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const Strea
         const int vend = pend[vp];
         for (; kb < vend; ++kb) {
             const int st = pos.st;
-            const uint32_t ph = pos.ph;
-            const bool ok = mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P.spin, g.abort);
+            pos.wait(full, P.spin, g.abort);
             const int lr0 = kb * rs_;
             const int rows = min(rs_, nrow - lr0);
             const float* stage = ring + (size_t)st * S.stage_floats;
-            for (int j = 0; ok && j < S.rpt; ++j) {
+            for (int j = 0; j < S.rpt; ++j) {
                 const int rr = tm.team + NTEAMS * j;
                 if (rr >= rows) break;
                 float4 x[VPT];
@@ -155,7 +154,7 @@ __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const Strea
                     }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[st]);
+            if (lane == 0) pos.release(empty, st);
             pos.next(S.stages);
         }
         // end of partition vp: teams' (max, sum) pairs merged in team order
@@ -423,12 +422,11 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
             const int vend = pend[vp];
             for (; kb < vend; ++kb) {
                 const int st = pos.st;
-                const uint32_t ph = pos.ph;
-                const bool ok = mbar_try_wait(&full[st], ph) || mbar_wait_bounded(&full[st], ph, P0.spin, g.abort);
+                pos.wait(full, P0.spin, g.abort);
                 const int lr0 = kb * rs_;
                 const int rows = min(rs_, nrow - lr0);
                 const float* stage = ring + (size_t)st * S.stage_floats;
-                for (int jr = 0; ok && jr < S.rpt; ++jr) {
+                for (int jr = 0; jr < S.rpt; ++jr) {
                     const int rr = tm.team + NTEAMS * jr;
                     if (rr >= rows) break;
                     const int lr = lr0 + rr;
@@ -534,7 +532,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
                     }
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[st]);
+                if (lane == 0) pos.release(empty, st);
                 pos.next(S.stages);
             }
             // end of partition vp: each active solve's column partials and row residual

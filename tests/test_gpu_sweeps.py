@@ -163,3 +163,38 @@ def test_rates_edges_and_scales(ctx, shape, scale):
     C2, _ = ctx.build_cost(R.contiguous(), inst.mu)
     assert torch.equal(C, C2)
     np.testing.assert_allclose(C.cpu().numpy(), 1.0 / (inst.mu * R_or), rtol=1e-6)
+
+
+def _times_out(ctx, call):
+    """`call` ends with OT_ETIMEOUT under a spin limit of one poll, time after time, and gives
+    what it gave before once the limit is back."""
+    from paper_1805_01559_gb300 import binding
+    want = call(3)
+    for _ in range(5):
+        ctx.set_spin_limit(1)
+        try:
+            with pytest.raises(binding.OTError) as e:
+                call(50)
+            assert e.value.status == binding.OT_ETIMEOUT
+        finally:
+            ctx.set_spin_limit(0)
+    for a, b in zip(want, call(3)):
+        assert torch.equal(a.f, b.f) and torch.equal(a.g, b.g)
+
+
+def _uniform(I, J):
+    C = torch.rand(I, J, device="cuda", generator=torch.Generator("cuda").manual_seed(J))
+    return C, torch.full((I,), 1.0 / I, device="cuda"), torch.full((J,), 1.0 / J, device="cuda")
+
+
+def test_timeout_of_wide_rows(ctx):
+    """Teams of two warps: a wait for a stage that gives up in one of them must not leave the
+    other at the team's barrier."""
+    t = _uniform(60000, 1280)
+    _times_out(ctx, lambda n: [ctx.solve_cost(*t, 0.1, tol=0.0, max_iter=n)])
+
+
+def test_timeout_of_wide_rows_multi(ctx):
+    """The same for three solves on one matrix."""
+    t = _uniform(60000, 800)
+    _times_out(ctx, lambda n: ctx.solve_cost_multi(*t, [0.1, 0.15, 0.2], tol=0.0, max_iter=n))
