@@ -468,7 +468,7 @@ struct SkShared {
     float errf[16];         // per-team row residuals
     double sh_sum[24][2];   // per-warp setup sums (up to 24 consumer warps)
     int s_dec, s_ok, s_bad;
-    int flags[2];                    // of a sweep, by parity: EXACT, BAD and LATE below
+    int flags[2];                    // of a sweep, by parity: the SK_ bits below
     unsigned long long s_err;        // total of the row residuals
     unsigned long long werr[16];     // per team, of the current partition
     volatile int s_stop;    // consumers -> producer: stop streaming
@@ -479,7 +479,11 @@ struct SkShared {
 enum : int {
     SK_EXACT = 1,  // some column's total has to be summed from the partials
     SK_BAD = 2,    // and one of those lost its mass
-    SK_LATE = 4,   // a wait for the totals gave up
+    // A wait for the totals gave up: for a thread's first columns, looked at after those, or for
+    // further ones, looked at after all.  Two bits: a thread may be waiting for further columns
+    // while another has yet to look at the first ones, and the CTA leaves as one.
+    SK_LATE = 4,
+    SK_LATER = 8,
 };
 
 // The CTAs that solve one instance together: nb CTAs, this one is number b.  `bar` counts
@@ -1665,12 +1669,12 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 }
                 ++n;
                 if ((n & 63) == 0 && ld_volatile_i32(g.abort) != DEV_OK) {
-                    atomicOr(flags, SK_LATE);
+                    atomicOr(flags, first ? SK_LATE : SK_LATER);
                     break;
                 }
                 if (n > P.spin) {
                     atomicCAS(g.abort, DEV_OK, DEV_ETIMEOUT);
-                    atomicOr(flags, SK_LATE);
+                    atomicOr(flags, first ? SK_LATE : SK_LATER);
                     break;
                 }
                 if (n > 256) __nanosleep(32);
@@ -1725,7 +1729,7 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
         if (exact) atomicOr(flags, SK_EXACT);
         bar_named(CONS_BAR, NC);
         const int fl = *(volatile int*)flags;
-        if (fl & SK_LATE) {
+        if (fl & SK_LATER) {
             if (tid == 0) s_stop = 1;
             return false;
         }

@@ -198,3 +198,11 @@ def test_timeout_of_wide_rows_multi(ctx):
     """The same for three solves on one matrix."""
     t = _uniform(60000, 800)
     _times_out(ctx, lambda n: ctx.solve_cost_multi(*t, [0.1, 0.15, 0.2], tol=0.0, max_iter=n))
+
+
+@pytest.mark.parametrize("shape", [(40000, 1500), (20000, 4100), (10000, 8192)])
+def test_timeout_with_many_columns_a_thread(ctx, shape):
+    """Rows so wide that a thread waits for its columns' totals in several rounds: a wait that
+    gives up in any of them ends the CTA as one."""
+    t = _uniform(*shape)
+    _times_out(ctx, lambda n: [ctx.solve_cost(*t, 0.1, tol=0.0, max_iter=n)])
