@@ -47,7 +47,7 @@ struct LoopState {
 //   [3 Jp, 4 Jp)    log2 q^_j as FP32 pairs
 //   [4 Jp, 4.5 Jp)  fixed-point shift S_j of column j (int)
 //   then 2 rows of Jp + 4 64-bit words: per-column fixed-point totals of the sweeps' column
-//   partials and their row residuals (word Jp); sweep s adds into row s mod 2.
+//   partials and their row residuals (words Jp and Jp + 2); sweep s adds into row s mod 2.
 //   then Jp FP32 pairs: G^0, later G^1, as the sweeps hold them.
 // The totals are sums of integers, the same in any order, so every CTA reads the same column
 // sums whatever the number of CTAs or the order in which partitions arrive.
@@ -470,6 +470,7 @@ struct SkShared {
     int s_dec, s_ok, s_bad;
     int flags[2];                    // of a sweep, by parity: the SK_ bits below
     unsigned long long s_err;        // total of the row residuals
+    unsigned long long err_was[2][2];  // a row's residual words when last complete (thread 0's)
     unsigned long long werr[16];     // per team, of the current partition
     volatile int s_stop;    // consumers -> producer: stop streaming
     uint32_t tmem;          // tensor-memory address of the column potentials (see G_to_tmem)
@@ -962,14 +963,14 @@ __device__ __forceinline__ unsigned long long row_updates(const float2* Fold, fl
         const float r = Fnew[lr].x;
         Fnew[lr] = df_sub(Fold[lr], log2_corr(r));
         const float x = Ps[lr] * fabsf(r - 1.0f) * 0x1p50f;
-        e += x < 0x1p52f ? __float2ull_rn(x) : 1ull << 52;
+        e += x < (float)FX_BROKEN ? __float2ull_rn(x) : FX_BROKEN;
     }
     const unsigned m = (1u << 18) - 1;
     const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)e & m);
     const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(e >> 18) & m);
     const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(e >> 36));
     e = a + ((unsigned long long)b << 18) + ((unsigned long long)c << 36);
-    return e < (1ull << 52) ? e : 1ull << 52;
+    return e < FX_BROKEN ? e : FX_BROKEN;
 }
 
 // The consumer warps' part of one solve (Algorithm 1 on the CTA's partitions, rows [r0, r1)):
@@ -1493,13 +1494,14 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     constexpr int UC = (4 * TT * VPT + NC - 1) / NC;  // columns a thread looks after: tid + NC u
     constexpr int CU = UC < 3 ? UC : 3;               // and how many at a time
     static_assert(UC <= 32, "one mask word");
-    unsigned long long prev[2][UC], prev_err[2] = {0ull, 0ull};  // the rows' words when last complete
+    unsigned long long prev[2][UC];  // the rows' words when last complete (the residual's: sh->err_was)
 #pragma unroll
     for (int u = 0; u < UC; ++u) prev[0][u] = prev[1][u] = 0ull;
-    if (tid == 0) sh->flags[0] = sh->flags[1] = 0;  // a barrier follows (G_to_tmem)
-    // the loop test's bound in the residual's units (totals stay below 2^FX_COUNT)
-    const double stop_d = stop_tol(P.tol) * 0x1p50;
-    const unsigned long long stop_units = stop_d < 0x1p56 ? (unsigned long long)stop_d : 1ull << FX_COUNT;
+    if (tid == 0) {
+        sh->flags[0] = sh->flags[1] = 0;  // a barrier follows (G_to_tmem)
+        sh->err_was[0][0] = sh->err_was[0][1] = sh->err_was[1][0] = sh->err_was[1][1] = 0ull;
+    }
+    const unsigned long long stop_units = fx_stop_units(stop_tol(P.tol) * 0x1p50);
     constexpr int RPP = rows_per_pass<TW, VPT, EUC>();
     // a step takes two blocks where a team's rows of one do not fill its passes, if the ring has
     // stages to spare for that
@@ -1589,8 +1591,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
                 unsigned long long e = 0ull;
 #pragma unroll
                 for (int t = 0; t < NTEAMS; ++t) e += sh->werr[t];
-                // at most 2^51 in all for a plan of unit mass; a broken plan's must not reach the count
-                atomicAdd(acc_s + Jp, FX_ONE + (e < (1ull << 52) ? e : 1ull << FX_TOP));
+                atomicAdd(acc_s + Jp, (unsigned long long)(FX_ONE + fx_err_low(e)));
+                atomicAdd(acc_s + Jp + 2, (unsigned long long)(FX_ONE + fx_err_high(e)));
             }
             if (tm.team >= HALF) {
 #pragma unroll
@@ -1621,8 +1623,11 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             for (int v = 0; v < VPT; ++v) acc[v][0] = acc[v][1] = 0ull;
             if (vp + 1 < v1) bar_named(CONS_BAR, NC);  // comb and werr are free again
         }
-        // a CTA without a partition counts itself into the residual word: it has read the other row
-        if (v0 == v1 && tid == 0) atomicAdd(acc_s + Jp, (unsigned long long)FX_ONE);
+        // a CTA without a partition counts itself into the residual words: it has read the other row
+        if (v0 == v1 && tid == 0) {
+            atomicAdd(acc_s + Jp, (unsigned long long)FX_ONE);
+            atomicAdd(acc_s + Jp + 2, (unsigned long long)FX_ONE);
+        }
         tmem_fence_before();  // this sweep's reads of G, before the barriers that precede its next copy
         // G^s_j = G^(s-1)_j + log2 q^_j - log2 s_j, every column in every CTA (FP32 pairs).  The
         // sum s_j is the fixed-point total T_j 2^-S_j; a column whose total is too large or too
@@ -1645,20 +1650,25 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             long long n = 0;
             for (;;) {  // until every addition due to this thread's words has arrived
                 bool all = true;
-                unsigned long long Ae = 0ull;
+                unsigned long long lo = 0ull, hi = 0ull;  // the residual's words
 #pragma unroll
                 for (int u = 0; u < CU; ++u) {
                     const int j = tid + (u0 + u) * NC;
                     A[u] = u0 + u < UC && j < J ? ld_relaxed_u64(acc_s + j) : was[u] + ((unsigned long long)fx_due_col(V) << FX_COUNT);
                 }
-                if (first && tid == 0) Ae = ld_relaxed_u64(acc_s + Jp);
+                if (first && tid == 0) {
+                    lo = ld_relaxed_u64(acc_s + Jp);
+                    hi = ld_relaxed_u64(acc_s + Jp + 2);
+                }
 #pragma unroll
                 for (int u = 0; u < CU; ++u) all = all && fx_complete(A[u], was[u], fx_due_col(V));
                 if (first && tid == 0) {
-                    all = all && fx_complete(Ae, prev_err[s & 1], fx_due_err(V, nb));
+                    unsigned long long* ew = sh->err_was[s & 1];
+                    all = all && fx_complete(lo, ew[0], fx_due_err(V, nb)) && fx_complete(hi, ew[1], fx_due_err(V, nb));
                     if (all) {
-                        sh->s_err = fx_value(Ae, prev_err[s & 1]);
-                        prev_err[s & 1] = Ae;
+                        sh->s_err = fx_err(fx_value(lo, ew[0]), fx_value(hi, ew[1]));
+                        ew[0] = lo;
+                        ew[1] = hi;
                     }
                 }
                 if (all) {

@@ -20,9 +20,9 @@ MODEL = r"""
 #include <vector>
 #include "sk_totals.h"
 using namespace ota;
-static const int W = 3, SWEEPS = 6;  // column words of a row, sweeps of a solve
+static const int NC = 3, W = NC + 2, SWEEPS = 6;  // columns, words of a row (two of the residual), sweeps
 static int V, nb;
-static uint64_t row[2][W + 1];
+static uint64_t row[2][W];
 static uint64_t value(int s, int v, int w) {  // of partition v in sweep s: up to the largest a word takes
     uint64_t h = (uint64_t)(s * 1000003 + v * 7919 + w * 104729 + 1) * 0x9e3779b97f4a7c15ull;
     return h % ((1ull << FX_TOP) + 1);
@@ -41,29 +41,29 @@ static int due_err() { return fx_due_err(V, nb); }
 #endif
 struct Cta {
     int v0, v1, s = 0, add = 0, wait = 0;
-    uint64_t was[2][W + 1] = {};
+    uint64_t was[2][W] = {};
     std::vector<int> order;  // in which it reads the words of a row
     bool done() const { return s == SWEEPS; }
     bool owns() const { return v0 < v1; }
     // one addition or one complete read; false when it has to wait
     bool step() {
         uint64_t* r = row[s & 1];
-        const int adds = owns() ? (v1 - v0) * (W + 1) : (bare ? 1 : 0);
+        const int adds = owns() ? (v1 - v0) * W : (bare ? W - NC : 0);
         if (add < adds) {
-            if (owns()) r[add % (W + 1)] += FX_ONE + value(s, v0 + add / (W + 1), add % (W + 1));
-            else r[W] += FX_ONE;
+            if (owns()) r[add % W] += FX_ONE + value(s, v0 + add / W, add % W);
+            else r[NC + add] += FX_ONE;
             ++add;
             return true;
         }
         const int w = order[wait];
         uint64_t& b = was[s & 1][w];
-        if (!fx_complete(r[w], b, w < W ? fx_due_col(V) : due_err())) return false;
+        if (!fx_complete(r[w], b, w < NC ? fx_due_col(V) : due_err())) return false;
         if (fx_value(r[w], b) != total(s, w)) {
             printf("wrong\n");
             exit(0);
         }
         b = r[w];
-        if (++wait == W + 1) {
+        if (++wait == W) {
             ++s;
             add = wait = 0;
         }
@@ -78,8 +78,8 @@ int main(int argc, char** argv) {
     std::vector<Cta> c(nb);
     for (int b = 0; b < nb; ++b) {
         cta_parts(V, b, nb, &c[b].v0, &c[b].v1);
-        for (int w = 0; w <= W; ++w) c[b].order.push_back(w);
-        for (int w = W; w > 0; --w) std::swap(c[b].order[w], c[b].order[rng() % (w + 1)]);
+        for (int w = 0; w < W; ++w) c[b].order.push_back(w);
+        for (int w = W - 1; w > 0; --w) std::swap(c[b].order[w], c[b].order[rng() % (w + 1)]);
     }
     for (;;) {
         bool moved = false, all = true;
@@ -115,21 +115,21 @@ int main(int argc, char** argv) {
 """
 
 
-@pytest.fixture(scope="module")
-def model(tmp_path_factory):
+def _compiled(folder, name, code, *flags):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
-    d = tmp_path_factory.mktemp("totals")
-    src = d / "model.cpp"
-    src.write_text(MODEL)
+    src, exe = folder / (name + ".cpp"), folder / name
+    src.write_text(code)
+    subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, *flags, str(src), "-o", str(exe)], check=True)
+    return lambda *a: subprocess.run([str(exe), *map(str, a)], check=True, capture_output=True, text=True,
+                                     timeout=120).stdout.strip()
 
-    def compiled(name, *flags):
-        exe = d / name
-        subprocess.run([cxx, "-O1", "-std=c++17", "-I", CSRC, *flags, str(src), "-o", str(exe)], check=True)
-        return lambda *a: subprocess.run([str(exe), *map(str, a)], check=True, capture_output=True, text=True,
-                                         timeout=120).stdout.strip()
-    return compiled("model"), compiled("without", "-DNO_BARE_COUNT")
+
+@pytest.fixture(scope="module")
+def model(tmp_path_factory):
+    d = tmp_path_factory.mktemp("totals")
+    return _compiled(d, "model", MODEL), _compiled(d, "without", MODEL, "-DNO_BARE_COUNT")
 
 
 # fewer partitions than CTAs, as many, more; 128 partitions, at which the 8-bit count of three
@@ -150,3 +150,44 @@ def test_model_sees_a_missing_count(model, V, nb, fails):
     """Without the bare count of CTAs that own no partition the same orders break the protocol."""
     _, run = model
     assert run(V, nb, 0, 0) == fails
+
+
+RESIDUAL = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "sk_totals.h"
+using namespace ota;
+// residual V nb e tol: V partitions of residual e (units) each; prints whether the words are
+// complete before and after the last addition, the total, and whether the loop test passes
+int main(int, char** argv) {
+    const int V = atoi(argv[1]), nb = atoi(argv[2]);
+    const uint64_t e = strtoull(argv[3], nullptr, 10), was = 0xfedcba9876543210ull;
+    uint64_t lo = was, hi = was;
+    int early = 0;
+    const int n = fx_due_err(V, nb);
+    for (int k = 0; k < n; ++k) {
+        early |= fx_complete(lo, was, n) || fx_complete(hi, was, n);
+        lo += FX_ONE + (k < V ? fx_err_low(e) : 0);
+        hi += FX_ONE + (k < V ? fx_err_high(e) : 0);
+    }
+    const bool full = fx_complete(lo, was, n) && fx_complete(hi, was, n);
+    const uint64_t t = fx_err(fx_value(lo, was), fx_value(hi, was));
+    printf("%d %d %llu %d", early, (int)full, (unsigned long long)t, (int)(t <= fx_stop_units(atof(argv[4]) * 0x1p50)));
+}
+"""
+
+UNIT = 1 << 50   # residual 1
+BROKEN = 1 << 52  # what a row that is not a number, infinite or 4 or more counts as
+
+
+@pytest.mark.parametrize("V,nb,e,tol,passes", [
+    (152, 152, 0, 0.0, True), (1, 1, 1, 0.0, False), (152, 152, 7, 1e-6, True), (152, 38, UNIT // 4, 0.3, False),
+    (1, 152, 2 * UNIT, 2.5, True), (1, 152, 2 * UNIT, 1.9, False), (1, 1, 2 * UNIT, float("inf"), True),
+    (1, 1, BROKEN, 0.3, False), (1, 1, BROKEN, 1e30, False), (152, 152, BROKEN, float("inf"), False),
+    (16, 16, BROKEN - 1, 10.0, False), (152, 152, BROKEN - 1, float("inf"), False), (152, 152, 16 * BROKEN, 100.0, False)])
+def test_residual_words(tmp_path, V, nb, e, tol, passes):
+    """The residual words hold any residuals exactly and never count an addition too many, and a
+    total that no plan of unit mass can have does not pass the loop test, whatever the tolerance."""
+    early, full, total, stop = map(int, _compiled(tmp_path, "residual", RESIDUAL)(V, nb, e, tol).split())
+    assert not early and full and total == V * e
+    assert bool(stop) == passes
