@@ -163,12 +163,16 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         }
     }
     F64_BARRIER();
+    // Written by then, if at all: from here on numerical failures are collected in `bad` and
+    // published with the residuals, so that every CTA takes the same decision on them.
+    if (__syncthreads_or(ld_volatile_i32(status) != DEV_OK)) return;
     const double sp = grid_total(P.part, nb, 0, &s_tot), sq = grid_total(P.part, nb, 1, &s_tot);
     if (!(fabs(sp - sq) <= 1e-5 * sp)) {
         if (b == 0 && tid == 0) atomicCAS(status, DEV_OK, DEV_EINVAL);
         return;  // the same decision in every CTA
     }
     const double inv_sp = 1.0 / sp, inv_sq = 1.0 / sq, lsp = log(sp);
+    int bad = 0;  // a potential that this thread formed is not finite
 
     // One row's sum over its team from the lanes' values (the whole block calls).
     auto row_sums = [&](double v) {
@@ -204,7 +208,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         if (tid < R && k * R + tid < I) {
             const int64_t ii = k * R + tid;
             const double fi = eps * (log(P.p[ii] * inv_sp) - (s_w[tid] + log(s_row[tid])));
-            if (!isfinite(fi)) atomicCAS(status, DEV_OK, F64_ENUMERIC);
+            bad |= !isfinite(fi);
             P.fb[I + ii] = fi;
         }
         __syncthreads();
@@ -222,7 +226,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
             s = block_sum(s, sh);
             if (tid == 0) {
                 const double v = log(P.q[j] * inv_sq) - (m + log(s));
-                if (!isfinite(v)) atomicCAS(status, DEV_OK, F64_ENUMERIC);
+                bad |= !isfinite(v);
                 P.gb[J + j] = eps * v;
             }
         }
@@ -255,7 +259,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
                 const int64_t ii = k * R + tid;
                 const double ph = P.p[ii] * inv_sp, w = ph / s_row[tid], fi = fprev[ii];
                 const double fn = fi + eps * log(w);
-                if (!isfinite(fn)) atomicCAS(status, DEV_OK, F64_ENUMERIC);
+                bad |= !isfinite(fn);
                 fcur[ii] = fn;
                 res += ph * fabs(expm1((fi - fn) * inv_eps));
                 s_w[tid] = w;
@@ -268,17 +272,23 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
             }
             __syncthreads();
         }
+        const int failed = __syncthreads_or(bad);  // the row updates', and the last column updates'
         if (warp == 0) {  // a tile's rows are updated by threads of warp 0
             res = warp_sum(res);
-            if (lane == 0) P.part[4 * b + 2] = res;
+            if (lane == 0) P.part[4 * b + 2] = failed ? NAN : res;
         }
         if (P.colp)
             for (int j = tid; j < J; j += F64_NT) P.colp[(int64_t)b * J + j].x = acc[j];
         F64_BARRIER();
         const double e = grid_total(P.part, nb, 2, &s_tot);
-        // the status is final for this test: the next write comes after the next barrier
-        const bool stop = (e <= P.tol) || (s - 1 >= P.max_iter) || ld_volatile_i32(status) != DEV_OK;
-        if (__syncthreads_or(stop)) {
+        if (isnan(e)) {  // some CTA has failed: every one leaves, and the caller's outputs stay as they are
+            if (b == 0 && tid == 0) {
+                P.st->iters = s - 1;
+                atomicCAS(status, DEV_OK, F64_ENUMERIC);
+            }
+            return;
+        }
+        if (e <= P.tol || s - 1 >= P.max_iter) {  // the same sum in every CTA
             if (b == 0 && tid == 0) {
                 P.st->iters = s - 1;
                 P.st->err = e;
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
             }
             if (lane == 0) {
                 const double gn = __ldcg(gprev + j) + eps * log(P.q[j] * inv_sq / c);
-                if (!isfinite(gn)) atomicCAS(status, DEV_OK, F64_ENUMERIC);
+                bad |= !isfinite(gn);
                 gcur[j] = gn;
             }
         }

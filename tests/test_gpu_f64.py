@@ -93,3 +93,29 @@ def test_fp64_rejects_unbalanced(ctx):
     with pytest.raises(binding.OTError) as e:
         ctx.solve_f64(_t(C), _t(np.full(10, 0.1)), _t(np.full(4, 0.5)), 0.1)
     assert e.value.status == binding.OT_EINVAL
+
+
+@pytest.mark.parametrize("shape", [(1000, 50), (40, 2881), (5, 3)])
+@pytest.mark.parametrize("lost", ["row", "column", "both"])
+def test_fp64_breakdown_is_one_decision(ctx, shape, lost):
+    """A device or an RRH without any link: every CTA leaves at the same loop test, time after
+    time, and the caller's outputs (a warm-start g among them) stay as they were."""
+    import ctypes
+
+    from paper_1805_01559_gb300 import binding
+    I, J = shape
+    C = np.random.Generator(np.random.PCG64(I + J)).uniform(0.0, 1.0, shape)
+    if lost in ("row", "both"):
+        C[I // 2] = np.inf
+    if lost in ("column", "both"):
+        C[:, J - 1] = np.inf
+    C, p, q = (torch.from_numpy(x).cuda() for x in (C, np.full(I, 1.0 / I), np.full(J, 1.0 / J)))
+    for _ in range(10):
+        r, f, g, _, load = ctx._result(I, J, C.device, False, True, None, None)
+        for x in (f, g, load):
+            x.fill_(7.0)
+        st = ctx._L.ot_assoc_solve_f64(ctx._h, binding._ptr(C), J, binding._ptr(p), binding._ptr(q), I, J, 0.1, 0.0, 20, 0,
+                                       ctypes.byref(r), binding._stream(None))
+        assert st == binding.OT_EINVAL and r.iters == 1
+        for x in (f, g, load):
+            assert bool((x == 7.0).all())
