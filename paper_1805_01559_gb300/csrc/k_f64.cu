@@ -10,7 +10,9 @@
 // (LSE with the maximum factored out), which no start can underflow.  Afterwards every plan
 // pi = exp((f + g - C) / eps) has exact columns and rows of at least min q^ of their mass, so
 // an iteration forms each pi_ij once: its row sums give f_i += eps log(p^_i / r_i), and the
-// column sums of pi_ij p^_i / r_i give g_j += eps log(q^_j / s_j).
+// column sums of pi_ij p^_i / r_i give g_j += eps log(q^_j / s_j).  Masses that differ by
+// hundreds of decades can still take r_i (down to p^_i min q^) or s_j below the range of a
+// double: a row or column whose sum is under F64_LOW is formed with its maximum factored out.
 //
 // What bounds it is the FP64 pipe: an exponential is some twenty instructions.  So a cell's
 // exponential is formed once an iteration (tiles of up to 8 rows in shared memory, summed by
@@ -37,6 +39,8 @@ namespace ota {
 static constexpr int F64_NT = 256;
 static constexpr int F64_NW = F64_NT / 32;
 enum : int { F64_ENUMERIC = -7 };
+// Terms lost below 2^-1022 are under 2^-122 of such a sum.
+static constexpr double F64_LOW = 0x1p-900;
 
 struct F64State {
     unsigned bar;
@@ -255,16 +259,44 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
                 }
             }
             row_sums(rs);
-            if (tid < nr) {
+            // row k R + tid, whose entries in T sum to s_row[tid] and stand for T e^m
+            auto update = [&](double m) {
                 const int64_t ii = k * R + tid;
                 const double ph = P.p[ii] * inv_sp, w = ph / s_row[tid], fi = fprev[ii];
-                const double fn = fi + eps * log(w);
+                const double fn = fi + eps * (log(w) - m);
                 bad |= !isfinite(fn);
                 fcur[ii] = fn;
                 res += ph * fabs(expm1((fi - fn) * inv_eps));
                 s_w[tid] = w;
+            };
+            const bool low = tid < nr && !(s_row[tid] >= F64_LOW);
+            if (tid < nr && !low) update(0.0);
+            if (__syncthreads_or(low)) {
+                const bool mine = r < nr && !(s_row[r] >= F64_LOW);  // this team's row
+                const double* row = P.C + (r < nr ? i : 0) * P.ld;
+                const double fi = r < nr ? fprev[i] : 0.0;
+                double m = -INFINITY;
+                if (mine)
+                    for (int j = tl; j < J; j += NTR) m = fmax(m, (fi + __ldcg(gprev + j) - row[j]) * inv_eps);
+                m = warp_maxd(m);
+                if (lane == 0) sh[warp] = m;
+                __syncthreads();
+                m = sh[r * WR];
+                for (int w = 1; w < WR; ++w) m = fmax(m, sh[r * WR + w]);
+                __syncthreads();
+                rs = 0.0;
+                if (mine)
+                    for (int j = tl; j < J; j += NTR) {
+                        const double t = exp((fi + __ldcg(gprev + j) - row[j]) * inv_eps - m);
+                        T[(size_t)r * J + j] = t;
+                        rs += t;
+                    }
+                row_sums(rs);
+                if (mine && tl == 0) s_w[r] = m;
+                __syncthreads();
+                if (low) update(s_w[tid]);
+                __syncthreads();
             }
-            __syncthreads();
             for (int j = tid; j < J; j += F64_NT) {
                 double a = acc[j];
                 for (int q = 0; q < nr; ++q) a = fma(T[(size_t)q * J + j], s_w[q], a);
@@ -307,8 +339,18 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
             } else {
                 c = acc[j];
             }
+            double m = -INFINITY;
+            const bool low = !(c >= F64_LOW);  // the same in the whole warp
+            if (low) {  // as in iteration 1, from the row potentials
+                for (int64_t i = lane; i < I; i += 32) m = fmax(m, (__ldcg(fcur + i) - P.C[i * P.ld + j]) * inv_eps);
+                m = warp_maxd(m);
+                c = 0.0;
+                for (int64_t i = lane; i < I; i += 32) c += exp((__ldcg(fcur + i) - P.C[i * P.ld + j]) * inv_eps - m);
+                c = warp_sum(c);
+            }
             if (lane == 0) {
-                const double gn = __ldcg(gprev + j) + eps * log(P.q[j] * inv_sq / c);
+                const double gn = low ? eps * (log(P.q[j] * inv_sq) - (m + log(c)))
+                                      : __ldcg(gprev + j) + eps * log(P.q[j] * inv_sq / c);
                 bad |= !isfinite(gn);
                 gcur[j] = gn;
             }

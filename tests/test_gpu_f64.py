@@ -119,3 +119,35 @@ def test_fp64_breakdown_is_one_decision(ctx, shape, lost):
         assert st == binding.OT_EINVAL and r.iters == 1
         for x in (f, g, load):
             assert bool((x == 7.0).all())
+
+
+@pytest.mark.parametrize("shape", [(2, 3), (9, 4), (300, 50), (40, 2881), (11, 8192)])
+@pytest.mark.parametrize("kind", ["row", "column"])
+def test_fp64_sums_below_the_range(ctx, shape, kind):
+    """Masses 200 decades apart.  row: a device of 1e-200 with one link, to an RRH of 1e-200 that
+    every other device reaches too: its row sum becomes 1e-400 after the first column update.
+    column: that device also has the only good link to an ordinary RRH, which takes it up to mass
+    1 and the next row update the small RRH down to 1e-400.  Iterates as the oracle's log-sum-exp
+    gives them: both in doubles, a few ulp an iteration on exponents of up to 1000, so 1e-10
+    relative as in the tests above."""
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 10007 + J))
+    eps = 0.01
+    C = rng.uniform(0.0, 0.5, shape)
+    p, q = rng.uniform(0.5, 1.5, I), rng.uniform(0.5, 1.5, J)
+    i, j, k = I - 1, J - 1, J // 2
+    C[i] = np.inf
+    C[i, j] = 0.0
+    if kind == "column":
+        C[:i, j] = np.inf
+        C[:i, k] = 700 * eps
+        C[i, k] = 0.0
+    p[i] = q[j] = 0.0
+    q *= p.sum() / q.sum()
+    p[i] = q[j] = 1e-200
+    n = 4
+    res = ctx.solve_f64(*(torch.from_numpy(x).cuda() for x in (C, p, q)), eps, tol=0.0, max_iter=n)
+    f, g, _, _ = oracle.sinkhorn(C, p, q, eps, 0.0, n)
+    assert res.iters == n
+    np.testing.assert_allclose(oracle.plan(C, res.f.cpu().numpy(), res.g.cpu().numpy(), eps), oracle.plan(C, f, g, eps),
+                               rtol=1e-10, atol=1e-300)
