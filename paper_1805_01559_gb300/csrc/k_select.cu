@@ -435,7 +435,7 @@ ot_status launch_median(ot_assoc_ctx* ctx, const float* x, int64_t rows, int64_t
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, rs_select, src, n, k1, k2, bracket, s1, s2, ss, cand, cap, 1LL << 24, out_dev);
+    e = cudaLaunchKernelEx(&cfg, rs_select, src, n, k1, k2, bracket, s1, s2, ss, cand, cap, ctx->spin_limit, out_dev);
     if (e != cudaSuccess) return cuda_error(ctx, e, "median launch");
     ctx->launches += 1;
     return OT_OK;

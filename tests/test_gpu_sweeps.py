@@ -206,3 +206,31 @@ def test_timeout_with_many_columns_a_thread(ctx, shape):
     gives up in any of them ends the CTA as one."""
     t = _uniform(*shape)
     _times_out(ctx, lambda n: [ctx.solve_cost(*t, 0.1, tol=0.0, max_iter=n)])
+
+
+@pytest.mark.parametrize("entry", ["median", "cost", "gains", "mobile"])
+def test_median_keeps_to_the_spin_limit(ctx, entry):
+    """The grid barriers of the median give up after the context's limit: every call that takes a
+    median then reports OT_ETIMEOUT, and gives what it gave before once the limit is back."""
+    from paper_1805_01559_gb300 import binding
+    I, J = 60000, 256
+    gen = torch.Generator("cuda").manual_seed(3)
+    x = torch.rand(I, J, device="cuda", generator=gen) + 0.5
+    P = torch.ones(J, device="cuda")
+    xy, v = torch.rand(I, 2, dtype=torch.float64, device="cuda", generator=gen) * 1e3, torch.zeros(I, 2, dtype=torch.float64, device="cuda")
+    rrh, shadow = torch.rand(J, 2, device="cuda", generator=gen) * 1e3, torch.zeros(I, J, device="cuda")
+    C = torch.empty(I, J, device="cuda")
+    call = {"median": lambda: ctx.median_f32(x.view(-1)),
+            "cost": lambda: ctx.build_cost(x, 1.0, eps_rel=0.1, C_out=C)[1],
+            "gains": lambda: ctx.build_cost_from_gains(x, P, 0.1, 1.0, 1.0, eps_rel=0.1, C_out=C)[1],
+            "mobile": lambda: ctx.build_cost_mobile(xy, v, rrh, shadow, P, 0.0, 1e3, 1e-13, 1.0, 1.0, C_out=C, eps_rel=0.1)[1]}[entry]
+    want = call()
+    ctx.set_spin_limit(1)
+    try:
+        for _ in range(3):
+            with pytest.raises(binding.OTError) as e:
+                call()
+            assert e.value.status == binding.OT_ETIMEOUT
+    finally:
+        ctx.set_spin_limit(0)
+    assert call() == want
