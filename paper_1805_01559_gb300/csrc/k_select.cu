@@ -22,6 +22,7 @@
 // cost and median of 50,000 x 800 take, and half of the 100 us of a 1000 x 50 cell.
 // Now one launch of 70 us there (18 us on 1000 x 50).
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -53,8 +54,9 @@ struct SelectState {            // zeroed before the launch
     int status;
     unsigned long long n_cand;  // entries found in [lo, hi]
     unsigned long long c_lo;    // entries found below lo
-    unsigned long long hist[RS_PASSES][2][RS_BINS];
+    unsigned long long hist[RS_PASSES][2][RS_BINS];  // a lone CTA keeps its counts to itself and has none of these
 };
+static constexpr size_t RS_LONE = offsetof(SelectState, hist);
 
 // The data a pass reads: a strided row-major view (rows x cols, leading dimension ld).
 // flat: the view is one contiguous run of rows * cols entries.
@@ -385,6 +387,10 @@ __global__ void __launch_bounds__(RS_NT, 1) rs_select(SelSrc src, int64_t n, lon
                 if (ok[e]) T.count(sh, x[e]);
         }
         __syncthreads();
+        if (nb == 1) {
+            T.pick([&](int t, int b) { return (unsigned long long)sh->h[t][b]; }, sh);
+            continue;
+        }
         for (int t = tid; t < nh * RS_BINS; t += RS_NT) {
             const unsigned c = (&sh->h[0][0])[t];
             if (c) atomicAdd(&st->hist[pass][0][0] + t, (unsigned long long)c);
@@ -411,19 +417,28 @@ ot_status launch_median(ot_assoc_ctx* ctx, const float* x, int64_t rows, int64_t
     const int bracket = n >= (1 << 20);  // below that, three passes over the data cost little
     // the bracket spans about 5% of the entries; more than n/16 means heavy ties
     const unsigned long long cap = bracket ? (unsigned long long)(n / 16) : 0ull;
+    int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nch + RS_NT - 1) / RS_NT, ctx->num_sms));
     const size_t off_cand = (size_t)round_up(sizeof(SelectState), 256);
-    char* ws = (char*)scratch(ctx, SLOT_SELECT, off_cand + sizeof(float) * (size_t)cap, &st);
+    size_t state = grid > 1 ? sizeof(SelectState) : RS_LONE;
+    char* ws = (char*)scratch(ctx, SLOT_SELECT, bracket ? off_cand + sizeof(float) * (size_t)cap : state, &st);
+    if (st == OT_ENOMEM && !bracket && grid > 1) {
+        // no room for the grid's histograms (98 KB) in the context's budget: one CTA, up to 2^20
+        // entries, does without
+        st = OT_OK;
+        grid = 1;
+        state = RS_LONE;
+        ws = (char*)scratch(ctx, SLOT_SELECT, state, &st);
+    }
     if (st) return st;
     SelectState* ss = (SelectState*)ws;
     float* cand = (float*)(ws + off_cand);
     const double sd = 0.5 * std::sqrt((double)SAMPLE);
     const long long s1 = (long long)(SAMPLE / 2 - 4.5 * sd), s2 = (long long)(SAMPLE / 2 + 4.5 * sd);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((nch + RS_NT - 1) / RS_NT, ctx->num_sms));
     if (allow_max_dynamic_smem((const void*)rs_select, RS_SMEM) != cudaSuccess) {
         cudaGetLastError();
         return set_error(ctx, OT_ECUDA, "median kernel: %zu bytes of shared memory refused", RS_SMEM);
     }
-    cudaError_t e = cudaMemsetAsync(ss, 0, sizeof(SelectState), s);
+    cudaError_t e = cudaMemsetAsync(ss, 0, state, s);
     if (e != cudaSuccess) return cuda_error(ctx, e, "median memset");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

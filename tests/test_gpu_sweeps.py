@@ -234,3 +234,19 @@ def test_median_keeps_to_the_spin_limit(ctx, entry):
     finally:
         ctx.set_spin_limit(0)
     assert call() == want
+
+
+@pytest.mark.parametrize("shape", [(1, 1), (7, 300), (1000, 50), (1023, 1024)])
+@pytest.mark.parametrize("kind", ["lognormal", "two_values"])
+def test_median_within_a_small_budget(shape, kind):
+    """Below 2^20 entries a median needs next to no scratch: a context with 8 KB of budget, which
+    has no room for the histograms of a whole grid, gives the exact median all the same."""
+    from paper_1805_01559_gb300 import binding
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 31 + J))
+    R = rng.lognormal(0.0, 2.0, shape) if kind == "lognormal" else np.where(rng.random(shape) < 0.5, 1.0, 2.0)
+    with binding.Context(0, hbm_budget_bytes=8192) as c:
+        C, eps = c.build_cost(torch.from_numpy(R.astype(np.float32)).cuda(), 1.0, eps_rel=1.0)
+        assert eps == oracle.median(C.cpu().numpy().astype(np.float64))
+        assert c.median_f32(C.view(-1)) == eps
+        assert c.scratch_bytes() <= 8192
