@@ -250,3 +250,19 @@ def test_median_within_a_small_budget(shape, kind):
         assert eps == oracle.median(C.cpu().numpy().astype(np.float64))
         assert c.median_f32(C.view(-1)) == eps
         assert c.scratch_bytes() <= 8192
+
+
+@pytest.mark.parametrize("shape", [(5, 2), (64, 51), (700, 50), (301, 800), (9, 8190)])
+@pytest.mark.parametrize("k,kw", [(-34, 0), (105, 0), (0, -26), (-34, -40)])
+def test_rates_do_not_depend_on_the_units(ctx, shape, k, kw):
+    """Gains and noise times a power of two: the same ratios, so the same rates and costs bit for
+    bit.  The bandwidth times one: the rates times it, and the costs divided by it.  (The factors
+    keep every product's low part a normal number or an exact subnormal.)"""
+    from paper_1805_01559_gb300 import instances as ins
+    I, J = shape
+    inst = ins.make_instance("t", I, J, 1000.0, I + J, hotspot=False, traffic_sigma=1.0, marginal="uniform")
+    G, P = torch.from_numpy(inst.G.astype(np.float32)).cuda(), torch.from_numpy(inst.P.astype(np.float32)).cuda()
+    R, R2 = torch.empty_like(G), torch.empty_like(G)
+    C, eps = ctx.build_cost_from_gains(G, P, inst.N0, inst.W_hz, inst.mu, eps_rel=0.05, R_out=R)
+    C2, eps2 = ctx.build_cost_from_gains(G * 2.0**k, P, inst.N0 * 2.0**k, inst.W_hz * 2.0**kw, inst.mu, eps_rel=0.05, R_out=R2)
+    assert torch.equal(R * 2.0**kw, R2) and torch.equal(C * 2.0**-kw, C2) and eps * 2.0**-kw == eps2
