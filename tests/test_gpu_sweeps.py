@@ -266,3 +266,30 @@ def test_rates_do_not_depend_on_the_units(ctx, shape, k, kw):
     C, eps = ctx.build_cost_from_gains(G, P, inst.N0, inst.W_hz, inst.mu, eps_rel=0.05, R_out=R)
     C2, eps2 = ctx.build_cost_from_gains(G * 2.0**k, P, inst.N0 * 2.0**k, inst.W_hz * 2.0**kw, inst.mu, eps_rel=0.05, R_out=R2)
     assert torch.equal(R * 2.0**kw, R2) and torch.equal(C * 2.0**-kw, C2) and eps * 2.0**-kw == eps2
+
+
+@pytest.mark.parametrize("noise", [1.0, 2.0**-40, 2.0**40])
+def test_rate_logarithm_error(ctx, noise):
+    """R = W log2(1 + SINR) with W = ln 2 and one RRH is log1p of a SINR that follows from the
+    documented FP32 steps.  Bound: 0.91 ulp, the error of the kernel's logarithm over every float of
+    [2^-50, 2^12] (evaluated on the host), here for random ones of every binade of [2^-49, 2^100],
+    the neighbourhoods of all powers of two and of all 1.5 2^k - 1, where its interval ends."""
+    rng = np.random.Generator(np.random.PCG64(5))
+    f32 = np.float32
+    x = [np.ldexp(rng.uniform(1.0, 2.0, 4096), e) for e in range(-49, 101)]
+    near = np.arange(-64, 65) * 2.0**-24
+    x += [np.ldexp(1.0 + near, e) for e in range(-48, 100)] + [1.5 * 2.0**e * (1.0 + near) - 1.0 for e in range(-1, 60)]
+    x = np.concatenate([np.concatenate(x), 0.5 + np.arange(-64, 65) * 2.0**-26])
+    x = x[x > 2.0**-49] * noise
+    x = x[x < 2.0**100].astype(f32)
+    G = torch.from_numpy(x[:, None].copy()).cuda()
+    R = ctx.build_rates(G, torch.ones(1, device="cuda"), noise, 0.69314718055994530942).cpu().numpy()[:, 0]
+    one = f32(noise)
+    T = x + one                      # the row total as an FP32 pair (an exact two-sum)
+    t = T - x
+    Tl = (x - (T - t)) + (one - t)
+    sinr = x / ((T - x) + Tl)        # own / interference, rounded to nearest
+    want = np.log1p(sinr.astype(np.longdouble))
+    ulp = np.ldexp(1.0, np.frexp(want.astype(np.float64))[1] - 24)
+    err = np.abs((R - want).astype(np.float64)) / ulp
+    assert err.max() <= 0.91, (err.max(), sinr[err.argmax()])
