@@ -293,3 +293,21 @@ def test_rate_logarithm_error(ctx, noise):
     ulp = np.ldexp(1.0, np.frexp(want.astype(np.float64))[1] - 24)
     err = np.abs((R - want).astype(np.float64)) / ulp
     assert err.max() <= 0.91, (err.max(), sinr[err.argmax()])
+
+
+@pytest.mark.parametrize("mu", [1.0, 3.0, 1e-6, 0.7, 2.0**29, 2.0**31, 2.0**-61])
+def test_cost_is_rounded_to_nearest(ctx, mu):
+    """C = (1/mu) / R as IEEE single precision divides, bit for bit: every mantissa of R in one
+    binade, random ones over every binade from subnormals to the largest (most of them inside the
+    range of the short form, some on either side), and the ends of that range."""
+    rng = np.random.Generator(np.random.PCG64(7))
+    f32 = np.float32
+    R = np.arange(0x3F800000, 0x40000000, dtype=np.uint32).view(f32)
+    bits = rng.integers(1, 0x7F800000, 1 << 22, dtype=np.uint32)
+    ends = np.concatenate([np.ldexp(1.0, e) * (1.0 + np.arange(-64, 64) * 2.0**-23) for e in (-51, 67)]).astype(f32)
+    R = np.concatenate([R, bits.view(f32), ends])
+    R = R[: R.size // 64 * 64].reshape(-1, 64)
+    C, _ = ctx.build_cost(torch.from_numpy(R).cuda(), mu)
+    with np.errstate(over="ignore", under="ignore"):
+        want = f32(1.0 / mu) / R
+    assert np.array_equal(C.cpu().numpy().view(np.uint32), want.view(np.uint32))
