@@ -64,7 +64,7 @@ struct F64Params {
     double* fb;     // [2][I] row potentials, unit mass (buffer s & 1 holds f^s)
     double* gb;     // [2][J] column potentials (buffer s & 1 holds g^s)
     double* part;   // [grid][4] per-CTA partial sums
-    double2* colp;  // [grid][J] per-CTA column sums, or null for a grid of one CTA
+    double2* colp;  // [min(grid, tiles)][J] column sums of the CTAs with tiles, or null for a grid of one CTA
     int rows;       // rows of a tile: 8, 4, 2 or 1
     F64State* st;
     // outputs
@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
     const int R = P.rows, WR = F64_NW / R;        // warps of a row's team
     const int r = warp / WR, tl = (warp % WR) * 32 + lane, NTR = 32 * WR;
     const int64_t ntile = (I + R - 1) / R;
+    const int nt = (int)min((int64_t)nb, ntile);  // CTAs with tiles; the others help with the columns
     double* T = tile;
     double* acc = tile + (size_t)R * J;
     double* acc2 = acc + J;
@@ -190,6 +191,16 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         }
     };
 
+    // log sum_i exp((f_i - C_ij) / eps) of column j, by one warp, in every lane
+    auto col_lse = [&](const double* f, int j) {
+        double m = -INFINITY, s = 0.0;
+        for (int64_t i = lane; i < I; i += 32) m = fmax(m, (__ldcg(f + i) - P.C[i * P.ld + j]) * inv_eps);
+        m = warp_maxd(m);
+        if (m > -INFINITY)
+            for (int64_t i = lane; i < I; i += 32) s += exp((__ldcg(f + i) - P.C[i * P.ld + j]) * inv_eps - m);
+        return m + log(warp_sum(s));
+    };
+
     // ---- iteration 1: log-sum-exp by rows, then by columns ----------------------------------
     for (int64_t k = b; k < ntile; k += nb) {
         const int64_t i = k * R + r;
@@ -220,7 +231,14 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
     F64_BARRIER();
     {
         const double* f1 = P.fb + I;
-        for (int j = b; j < J; j += nb) {
+        // a CTA a column, or a warp where every warp of the grid has one
+        const bool by_warp = J >= nb * F64_NW;
+        for (int j = b + nb * warp; by_warp && j < J; j += nb * F64_NW) {
+            const double v = log(P.q[j] * inv_sq) - col_lse(f1, j);
+            bad |= !isfinite(v);
+            if (lane == 0) P.gb[J + j] = eps * v;
+        }
+        for (int j = b; !by_warp && j < J; j += nb) {
             double m = -INFINITY;
             for (int64_t i = tid; i < I; i += F64_NT) m = fmax(m, (__ldcg(f1 + i) - P.C[i * P.ld + j]) * inv_eps);
             m = block_max(m, sh);
@@ -309,7 +327,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
             res = warp_sum(res);
             if (lane == 0) P.part[4 * b + 2] = failed ? NAN : res;
         }
-        if (P.colp)
+        if (P.colp && b < nt)
             for (int j = tid; j < J; j += F64_NT) P.colp[(int64_t)b * J + j].x = acc[j];
         F64_BARRIER();
         const double e = grid_total(P.part, nb, 2, &s_tot);
@@ -334,22 +352,15 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         for (int j = b + nb * warp; j < J; j += nb * F64_NW) {
             double c = 0.0;
             if (P.colp) {
-                for (int bb = lane; bb < nb; bb += 32) c += __ldcg(&P.colp[(int64_t)bb * J + j].x);
+                for (int bb = lane; bb < nt; bb += 32) c += __ldcg(&P.colp[(int64_t)bb * J + j].x);
                 c = warp_sum(c);
             } else {
                 c = acc[j];
             }
-            double m = -INFINITY;
-            const bool low = !(c >= F64_LOW);  // the same in the whole warp
-            if (low) {  // as in iteration 1, from the row potentials
-                for (int64_t i = lane; i < I; i += 32) m = fmax(m, (__ldcg(fcur + i) - P.C[i * P.ld + j]) * inv_eps);
-                m = warp_maxd(m);
-                c = 0.0;
-                for (int64_t i = lane; i < I; i += 32) c += exp((__ldcg(fcur + i) - P.C[i * P.ld + j]) * inv_eps - m);
-                c = warp_sum(c);
-            }
+            const bool low = !(c >= F64_LOW);  // the same in the whole warp: as in iteration 1
+            const double lse = low ? col_lse(fcur, j) : 0.0;
             if (lane == 0) {
-                const double gn = low ? eps * (log(P.q[j] * inv_sq) - (m + log(c)))
+                const double gn = low ? eps * (log(P.q[j] * inv_sq) - lse)
                                       : __ldcg(gprev + j) + eps * log(P.q[j] * inv_sq / c);
                 bad |= !isfinite(gn);
                 gcur[j] = gn;
@@ -400,7 +411,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         er = warp_sum(er);
         if (lane == 0) P.part[4 * b + 0] = er;
     }
-    if (P.colp)
+    if (P.colp && b < nt)
         for (int j = tid; j < J; j += F64_NT) P.colp[(int64_t)b * J + j] = make_double2(acc[j], acc2[j]);
     F64_BARRIER();
     {
@@ -408,7 +419,7 @@ __global__ void __launch_bounds__(F64_NT) sk_solve64(F64Params P) {
         for (int j = b + nb * warp; j < J; j += nb * F64_NW) {
             double c = 0.0, h = 0.0;
             if (P.colp) {
-                for (int bb = lane; bb < nb; bb += 32) {
+                for (int bb = lane; bb < nt; bb += 32) {
                     const double2 v = __ldcg(&P.colp[(int64_t)bb * J + j]);
                     c += v.x;
                     h += v.y;
@@ -464,10 +475,14 @@ ot_status launch_solve_f64(ot_assoc_ctx* ctx, const SolveArgs64& a, SolveSummary
     ot_status st = OT_OK;
     const int64_t I = a.I;
     const int J = a.J;
-    // rows of a tile: as many as fit with the two rows of column sums (8 up to 2,896 columns)
+    // rows of a tile: as many as fit with the two rows of column sums (8 up to 2,896 columns), and
+    // fewer where that gives more SMs a tile and leaves a lane two columns of its row or more
     int rows = F64_NW;
     const size_t budget = 232448 - 2048;  // 227 KB per block minus static shared memory
-    while (rows > 1 && sizeof(double) * (size_t)(rows + 2) * J > budget) rows /= 2;
+    auto tiles = [&](int r) { return (I + r - 1) / r; };
+    while (rows > 1 && (sizeof(double) * (size_t)(rows + 2) * J > budget ||
+                        (tiles(rows / 2) <= ctx->num_sms && J >= 2 * 32 * (2 * F64_NW / rows))))
+        rows /= 2;
     const size_t smem = sizeof(double) * (size_t)(rows + 2) * J;
     if (allow_max_dynamic_smem((const void*)sk_solve64, smem) != cudaSuccess) {
         cudaGetLastError();
@@ -478,7 +493,10 @@ ot_status launch_solve_f64(ot_assoc_ctx* ctx, const SolveArgs64& a, SolveSummary
         cudaGetLastError();
         return set_error(ctx, OT_ECUDA, "FP64 solver cannot be resident");
     }
-    int grid = (int)std::max<int64_t>(1, std::min<int64_t>((I + rows - 1) / rows, (int64_t)ctx->num_sms));
+    // a CTA a tile, and enough for a warp a column: 20 iterations on 1 x 8,192 take 0.32 ms; with the
+    // tiles' CTAs alone they took 42 (one CTA, its warps walking 1,024 columns each), and 6 with a
+    // warp a row and a warp a column.  64 x 512: 0.39, 1.73 and 1.20 ms.
+    int grid = (int)std::min<int64_t>(std::max<int64_t>(tiles(rows), (J + F64_NW - 1) / F64_NW), ctx->num_sms);
     double* fb = (double*)scratch(ctx, SLOT_F, sizeof(double) * 2 * (size_t)I, &st);
     if (st) return st;
     double* gb = (double*)scratch(ctx, SLOT_G, sizeof(double) * 2 * (size_t)round_up(J, 4), &st);
@@ -493,7 +511,7 @@ ot_status launch_solve_f64(ot_assoc_ctx* ctx, const SolveArgs64& a, SolveSummary
     // alone keeps its sums in shared memory)
     double2* colp = nullptr;
     while (grid > 1) {
-        colp = (double2*)scratch(ctx, SLOT_COLPART, sizeof(double2) * (size_t)grid * J, &st);
+        colp = (double2*)scratch(ctx, SLOT_COLPART, sizeof(double2) * (size_t)std::min<int64_t>(grid, tiles(rows)) * J, &st);
         if (!st) break;
         if (st != OT_ENOMEM) return st;
         st = OT_OK;

@@ -151,3 +151,40 @@ def test_fp64_sums_below_the_range(ctx, shape, kind):
     assert res.iters == n
     np.testing.assert_allclose(oracle.plan(C, res.f.cpu().numpy(), res.g.cpu().numpy(), eps), oracle.plan(C, f, g, eps),
                                rtol=1e-10, atol=1e-300)
+
+
+# Where the rows of a tile, the grid, or the way a column is walked change: one row, fewer tiles than
+# column CTAs, the widths from which a tile takes 4, 2 and 1 rows, as many rows as SMs and one more,
+# the width from which every warp has a column.
+@pytest.mark.parametrize("shape", [(1, 1), (1, 9), (1, 8192), (2, 300), (7, 127), (7, 128), (33, 255), (33, 256), (64, 511),
+                                   (64, 512), (152, 512), (153, 512), (304, 600), (305, 600), (152, 1215), (152, 1216),
+                                   (3, 7201)])
+def test_fp64_wide_and_short(ctx, shape):
+    """Against the oracle after 4 iterations, 1e-10 relative as above."""
+    I, J = shape
+    rng = np.random.Generator(np.random.PCG64(I * 10007 + J))
+    C = rng.uniform(0.0, 1.0, shape)
+    p, q = rng.lognormal(0.0, 1.0, I), rng.uniform(0.5, 1.5, J)
+    q *= p.sum() / q.sum()
+    res = ctx.solve_f64(*(torch.from_numpy(x).cuda() for x in (C, p, q)), 0.05, tol=0.0, max_iter=4)
+    f, g, _, _ = oracle.sinkhorn(C, p, q, 0.05, 0.0, res.iters)
+    np.testing.assert_allclose(oracle.plan(C, res.f.cpu().numpy(), res.g.cpu().numpy(), 0.05), oracle.plan(C, f, g, 0.05),
+                               rtol=1e-10, atol=1e-300)
+    cost, rho, _, _ = oracle.finalize(C, f, g, p, q, 0.05)
+    assert res.transport_cost == pytest.approx(cost, rel=1e-12)
+    np.testing.assert_allclose(res.rrh_load.cpu().numpy(), rho, rtol=1e-12)
+
+
+def test_fp64_one_row_uses_the_chip(ctx):
+    """One device and 8,192 RRHs: 20 iterations take 42 ms if the one CTA with a row does all the
+    columns too, and 6 with a warp a column over every SM."""
+    import time
+    C = torch.rand(1, 8192, dtype=torch.float64, device="cuda")
+    p, q = torch.ones(1, dtype=torch.float64, device="cuda"), torch.full((8192,), 1.0 / 8192, dtype=torch.float64, device="cuda")
+    best = 1e9
+    for _ in range(5):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        ctx.solve_f64(C, p, q, 0.1, tol=0.0, max_iter=20)
+        best = min(best, time.perf_counter() - t0)
+    assert best < 15e-3
