@@ -572,6 +572,8 @@ __device__ __forceinline__ void cta_col_sum(float* comb, const float4 (&acc)[VPT
 template <int TW, int VPT>
 constexpr int tmem_cols() {
     constexpr int n = 8 * VPT * (TW == 8 ? 2 : 1);
+    // lane positions have to repeat with the warp quarters, and the columns to fit what is allocated
+    static_assert((TW == 1 || TW == 2 || TW == 4 || TW == 8) && n <= 128, "columns of tensor memory");
     return n <= 32 ? 32 : (n <= 64 ? 64 : 128);
 }
 template <int TW, int VPT>
