@@ -198,7 +198,7 @@ __device__ __noinline__ bool bt_instance(const BInst& D, BRes* out, int* abort, 
     }
     __syncthreads();  // the producer has drained its copies
     if (warp == 0) tmem_free(sh->tmem, tmem_cols<1, VPT>());
-    if (ld_volatile_i32(abort) != DEV_OK) return false;
+    if (__syncthreads_or(ld_volatile_i32(abort) != DEV_OK)) return false;
     if (s_res == 0) {  // the instance failed (the same in every CTA of the group)
         if (rank == 0 && threadIdx.x == 0) {
             out->iters = 0;

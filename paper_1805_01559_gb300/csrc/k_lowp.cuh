@@ -281,7 +281,7 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
         if (tid == 0 && sh->s_bad) atomicCAS(status, DEV_OK, DEV_EINVAL);
     }
     LP_BARRIER();
-    if (ld_volatile_i32(status) != DEV_OK) {
+    if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {
         if (tid == 0) s_stop = 1;
         return false;
     }
@@ -529,7 +529,7 @@ __device__ __forceinline__ bool lp_consumers(const LpParams& P, const StreamCfg&
             return true;
         }
         LP_BARRIER();
-        if (ld_volatile_i32(status) != DEV_OK) {
+        if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {
             if (tid == 0) s_stop = 1;
             return false;
         }

@@ -103,6 +103,22 @@ __device__ __forceinline__ void bar_named(int id, int n) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// The same, and whether any of the n threads says x: all get one answer.  A status word that other
+// CTAs may be writing is looked at through this (or by one thread for all): threads that read it
+// one by one can disagree, and those that stay would wait for the ones that left, without limit.
+__device__ __forceinline__ bool bar_named_or(int id, int n, bool x) {
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.s32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((int)x), "r"(id), "r"(n)
+        : "memory");
+    return r != 0;
+}
+
 __device__ __forceinline__ float& comp(float4& v, int c) {
     return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
 }

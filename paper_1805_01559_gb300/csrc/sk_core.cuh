@@ -1019,13 +1019,13 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
             return false;                                                                          \
         }                                                                                          \
     } while (0)
-// After a barrier that no status write can overtake (the next write comes after the next
-// barrier): leave when the instance failed.  Only needed when a failed instance does not
-// also end every wait (batched launches keep the abort word apart from instance status).
+// After a barrier, leave when the instance failed before it.  Only needed when a failed instance
+// does not also end every wait (batched launches keep the abort word apart from instance status).
+// A write after the barrier that a CTA already sees here makes all CTAs leave before the next one.
 #define OTA_BARRIER_CHECK()                                                                        \
     do {                                                                                           \
         OTA_BARRIER();                                                                             \
-        if (g.abort != status && ld_volatile_i32(status) != DEV_OK) {                              \
+        if (g.abort != status && bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {  \
             if (tid == 0) s_stop = 1;                                                              \
             return false;                                                                          \
         }                                                                                          \

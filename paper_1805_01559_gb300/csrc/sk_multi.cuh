@@ -254,7 +254,7 @@ __device__ __forceinline__ bool ms_first_sweep(const SolveParams& P, const Strea
         }
     }
     if (!grid_barrier_named(g.bar, (unsigned)nb * ++g.gen, g.abort, P.spin, CONS_BAR, NC, &sh->s_ok)) return false;
-    if (ld_volatile_i32(g.status) != DEV_OK) return false;
+    if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(g.status) != DEV_OK)) return false;
     load_G_smem(P.G + Jp, J, Jp, Gs, tid, NC);
     bar_named(CONS_BAR, NC);
     return true;
@@ -335,7 +335,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
         if (tid == 0 && sh->s_bad) atomicCAS(status, DEV_OK, DEV_EINVAL);
     }
     OTA_MS_BARRIER();
-    if (ld_volatile_i32(status) != DEV_OK) {
+    if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {
         if (tid == 0) s_stop = 1;
         return false;
     }
@@ -610,7 +610,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
         if (tid == 0) sh->s_dec = 0;
         if (!active) break;
         OTA_MS_BARRIER();
-        if (ld_volatile_i32(status) != DEV_OK) {
+        if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {
             if (tid == 0) s_stop = 1;
             return false;
         }
@@ -618,7 +618,7 @@ __device__ __forceinline__ bool ms_consumers(const MultiParams& M, const StreamC
             if ((active >> s) & 1u) load_G_smem(M.P[s].G + (it & 1) * Jp, J, Jp, Gbase + (size_t)2 * s * Jp, tid, NC);
         bar_named(CONS_BAR, NC);
     }
-    if (ld_volatile_i32(status) != DEV_OK) {
+    if (bar_named_or(CONS_BAR, NC, ld_volatile_i32(status) != DEV_OK)) {
         if (tid == 0) s_stop = 1;
         return false;
     }

@@ -274,3 +274,27 @@ def test_batch_timeout_is_reported(ctx):
         ctx.set_spin_limit(0)
     res = ctx.solve_batched(items)
     assert res[0].status in (binding.OT_OK, binding.OT_NOT_CONVERGED)
+
+
+def test_failed_instances_end_alone_time_after_time(ctx):
+    """Instances that fail in the set-up (unbalanced marginals) and in the first sweep (an RRH
+    without links) among sound ones, on groups of every size that the rounds hold: the same
+    outcome each time, and the sound ones bit for bit those of a batch of their own."""
+    from paper_1805_01559_gb300 import binding
+    rng = _rng(31)
+    shapes = [(700, 52), (3000, 130), (200, 8), (9000, 400), (64, 1000)]
+    good = [_inst(rng, I, J, eps=0.1, tol=1e-6, max_iter=200)[0] for I, J in shapes]
+    bad = [_inst(rng, I, J, eps=0.1, tol=1e-6, max_iter=200)[0] for I, J in shapes * 2]
+    for k, x in enumerate(bad):
+        if k % 2:
+            x.q = x.q * 2.0
+        else:
+            x.C[:, 1] = float("inf")
+    want = ctx.solve_batched(good)
+    want = [(r.iters, x.f.clone(), x.g.clone()) for r, x in zip(want, good)]
+    mixed = [y for k, x in enumerate(good) for y in (bad[2 * k], x, bad[2 * k + 1])]
+    for _ in range(20):
+        res = ctx.solve_batched(mixed)
+        for k, (it, f, g) in enumerate(want):
+            assert [res[3 * k].status, res[3 * k + 2].status] == [binding.OT_EINVAL] * 2
+            assert res[3 * k + 1].iters == it and torch.equal(good[k].f, f) and torch.equal(good[k].g, g)
