@@ -18,8 +18,8 @@
 // exponential is formed once an iteration (tiles of up to 8 rows in shared memory, summed by
 // row, then by column), by every SM, and per-row logarithms are taken a tile at a time.  With
 // two passes over the row and two over the column (the column's by one warp a column, 50 of
-// them on 1000 x 50) an iteration took 97 us and the solve of 26 iterations 2.57 ms; it takes
-// 0.47 ms now, with the same error (1e-14) against a plain FP64 reference.
+// them on 1000 x 50) an iteration took 97 us and the solve of 26 iterations 2.50 ms; it takes
+// 0.46 ms now, with the same error (1e-14) against a plain FP64 reference.
 //
 // As in the FP32 solver, the row update of iteration s also gives the row residual of the plan
 // of iteration s - 1 (p^_i |exp((f_i^(s-1) - f_i^s) / eps) - 1|), the loop test ("while

@@ -247,8 +247,8 @@ __device__ __forceinline__ void euclid_row(float2 d, const float* rx, const floa
 // The sweeps read a CTA's rows round after round, so a matrix larger than L2 (129 MB) would
 // leave nothing of itself there for the next sweep.  The first L2_KEEP bytes of a CTA's rows
 // (80 MB over 152 SMs, 5/8 of L2) keep the normal eviction priority and the rest is marked to
-// be evicted first, so the kept part survives and is read from L2.  50,000 x 800 (160 MB):
-// 954 -> 880 us a solve, 48 ragged instances 12.7 -> 12.4 ms.  Kept parts from 60 to 100 MB and
+// be evicted first, so the kept part survives and is read from L2.  By itself that took 8% off a
+// 50,000 x 800 solve (160 MB) and 2% off 48 ragged instances.  Kept parts from 60 to 100 MB and
 // the persisting priority (evict_last) instead of the normal one differ by 3% at most; the
 // persisting one would hold L2 against whatever runs next.
 static constexpr int64_t L2_KEEP = 80000000 / 152;
@@ -567,8 +567,8 @@ __device__ __forceinline__ void cta_col_sum(float* comb, const float4 (&acc)[VPT
 // The sweep reads G (eight bytes a column) once per row: from shared memory that was two thirds
 // of its shared-memory wavefronts (84 a row of 800 columns, with 25 more for the copy that
 // fills the ring), the busiest unit of the sweep.  Out of tensor memory the sweep of a
-// 50,000 x 800 solve takes 41,000 cycles a CTA instead of 46,600, and the whole solve 0.98 ms
-// instead of 1.00 (1.04 before the packed arithmetic); 100,000 x 1,536: 2.50 ms against 3.03.
+// 50,000 x 800 solve takes 41,000 cycles a CTA instead of 46,600 (2% of the solve when the sync
+// still hid most of it), and a 100,000 x 1,536 solve 17% less.
 template <int TW, int VPT>
 constexpr int tmem_cols() {
     constexpr int n = 8 * VPT * (TW == 8 ? 2 : 1);
@@ -873,10 +873,9 @@ __device__ __forceinline__ void team_sum_rows(float (&v)[R], float* red, int nte
 }
 
 // Rows a team takes at once.  Two rows of up to 6 chunks a lane fit the registers (128 a
-// thread); at 7 chunks the second row spills (50,000 x 800: 1.01 ms with two rows, 0.98 with
-// one).  Wider teams stay at one: their rows come from HBM, not L2, at the sizes that matter,
-// and two rows took 2.55 ms against 2.50 on 100,000 x 1,536.  1000 x 50 takes 245 us with two
-// rows, 255 with one.
+// thread); at 7 chunks the second row spills (50,000 x 800: 3% slower with two rows).  Wider
+// teams stay at one: their rows come from HBM, not L2, at the sizes that matter (100,000 x 1,536:
+// 2% slower with two).  1000 x 50 is 4% faster with two rows.
 template <int TW, int VPT, bool EUC>
 __host__ __device__ constexpr int rows_per_pass() {
     return EUC || TW > 1 || VPT > 6 ? 1 : 2;
@@ -888,7 +887,7 @@ __host__ __device__ constexpr int rows_per_pass() {
 // Bound by instruction issue and by the latency of a row's chain (shared-memory loads, ex2,
 // the team sum, the update) once C streams: two rows in flight hide one chain behind the
 // other and share the loads of G, and packed arithmetic halves the instructions of the
-// exponent and the accumulation (50,000 x 800: 1.04 -> 1.00 ms, 100,000 x 1,536: 3.98 -> 3.03,
+// exponent and the accumulation (by itself 4% of a 50,000 x 800 solve, and 24% at 100,000 x 1,536
 // with the chunk count of a lane fitted to the row for wide teams too).  Every operation
 // rounds as for one row at a time, so results are the same bit for bit.
 template <int TW, int VPT, bool EUC, int R>
@@ -955,8 +954,7 @@ __device__ __forceinline__ void sweep_rows(const float* (&row)[R], const float2 
 // units of 2^-FX_ERR, an integer so that its order does not matter.  Called by the warp that
 // stored the sums.  Done for every row by a whole warp inside the sweep, this took 270 of the
 // 1,370 cycles of a row of 800 columns, and FP64 in the loop test 1,000 cycles of every sync;
-// without both 1000 x 50 went from 207 to 190 us, 5,000 x 128 warm from 155 to 144, 48 ragged
-// instances from 13.1 to 12.7 ms.
+// without both 1000 x 50 took 8% less, 5,000 x 128 warm 7%, 48 ragged instances 3%.
 __device__ __forceinline__ unsigned long long row_updates(const float2* Fold, float2* Fnew, const float* Ps, int lr0,
                                                           int step, int end, int lane) {
     unsigned long long e = 0ull;
@@ -1491,8 +1489,8 @@ __device__ __forceinline__ bool sk_consumers(const SolveParams& P, const StreamC
     // The sync bounds small instances (it is half of an iteration up to 20,000 x 400) and idles
     // HBM in large ones.  A grid barrier cost three dependent trips through L2 (the adds have to
     // land before the arrival is released, the arrival, the totals); waiting on the counted
-    // totals costs one: 1000 x 50 245 -> 206 us, 5,000 x 128 warm 169 -> 155, 12,347 x 1,021
-    // packed 444 -> 426, 50,000 x 800 982 -> 964.
+    // totals costs one: by itself 16% of a 1000 x 50 solve, 8% of 5,000 x 128 warm, 4% of
+    // 12,347 x 1,021 packed, 2% of 50,000 x 800.
     constexpr int UC = (4 * TT * VPT + NC - 1) / NC;  // columns a thread looks after: tid + NC u
     constexpr int CU = UC < 3 ? UC : 3;               // and how many at a time
     static_assert(UC <= 32, "one mask word");
